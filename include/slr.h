@@ -103,7 +103,7 @@ typedef struct {
     int32_t band_slots;     /* shared-memory buffers the band solve streams its factor
                                through: 2..8; 0 = automatic                              */
     int32_t band_threads;   /* threads per band-solve CTA: 512 (one CTA per SM), 256 (two
-                               per SM, for more CTAs than SMs) or 32 (one warp per
+                               per SM, for more CTAs than SMs) or 32 (four warps per
                                subdomain, for planes of at most 64 rows in one slice;
                                other planes take the automatic choice); 0 = automatic
                                (32 where it applies)                                     */
@@ -167,7 +167,7 @@ typedef struct {
     int32_t tuned;               /* 1: the three above were chosen by timing (autotune)    */
     double tune_seconds;         /* time the tuning took (0 when taken from the cache)      */
     int32_t band_threads;        /* threads per band-solve CTA (256: two subdomains per SM;
-                                    32: a warp per subdomain)                               */
+                                    32: four warps per subdomain)                             */
     int32_t c_top_levels;        /* levels of C's factor solved with the explicit inverse   */
     int32_t c_top_positions;     /* interface positions in those levels                     */
     int64_t c_top_entries;       /* stored entries of that inverse (each layout)            */

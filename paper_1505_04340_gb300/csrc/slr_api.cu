@@ -143,6 +143,7 @@ slr_status upload_operator(slr_handle h, DevOperator<T>& op, bool with_band) {
     const int32_t r = std::max(1, h->opts.nrhs_max);
     CS(upload_band(h, &op.band));
     if (with_band) CS(upload(h, &op.bfac, hs.bfac));
+    op.bfac_len = hs.bfac_len;
     op.band_G = hs.band_G;
     op.band_nbuf = h->opts.band_slots;
     op.band_nt = hs.band_nt;
@@ -582,6 +583,7 @@ slr_status run_lanczos_deflated(slr_handle h, int32_t k_add, int32_t steps, cuda
         dfree(h, op.band, hs.band.size());
         CS(upload_band(h, &op.band));
         CS(upload(h, &op.bfac, hs.bfac));
+        op.bfac_len = hs.bfac_len;
         op.band_G = hs.band_G;
     }
     const int32_t mk = std::max(m, k);
@@ -810,6 +812,7 @@ slr_status device_band_pack(slr_handle h, DevOperator<T>& op, cudaStream_t st) {
     int32_t cmax = 0;
     for (const BandBlock& b : hs.band) cmax = std::max(cmax, b.c);
     CS(dalloc(h, &op.bfac, (size_t)hs.bfac_len));
+    op.bfac_len = hs.bfac_len;
     CK(cudaMemsetAsync(op.bfac, 0, sizeof(T) * hs.bfac_len, st));
     CK(launch_band_pack<T>(op.band, hs.p, cmax, hs.band_G, h->bf_scr, h->bf_soff, op.bfac, hs.indefinite, st));
     return SLR_OK;
@@ -831,6 +834,7 @@ slr_status repack_band(slr_handle h, DevOperator<T>& op, int32_t G) {
     if (h->bf_scr) CS(device_band_pack<T>(h, op, h->stream));
     else CS(upload(h, &op.bfac, hs.bfac));
     CK(cudaStreamSynchronize(h->stream));
+    op.bfac_len = hs.bfac_len;
     op.band_G = hs.band_G;
     return SLR_OK;
 }
@@ -868,7 +872,7 @@ slr_status autotune(slr_handle h, DevOperator<T>& op, cudaStream_t st) {
             if (G != hs.band_G) CS(repack_band<T>(h, op, G));
             for (int32_t nt : {512, 256, 32})
                 for (int32_t slots : {2, 3, 4}) {
-                    // the warp kernel: planes of at most 64 rows in one slice, its own ring
+                    // the narrow-plane kernel: planes of at most 64 rows in one slice, its own ring
                     if (nt == 32 && (G != 1 || hs.wmax > 64 || slots != 2)) continue;
                     op.band_nbuf = slots;
                     op.band_nt = nt;
@@ -969,7 +973,7 @@ slr_status setup_impl(slr_handle h, int32_t n, const int32_t* rowptr, const int3
         if (dev_band) host_band_layout(hs, G);
         else CS(host_band_factor(hs, G));
         // more CTAs than SMs would run in two waves: 256-thread CTAs put two subdomains on an SM;
-        // planes of at most 64 rows in one slice take a warp per subdomain
+        // planes of at most 64 rows in one slice take the narrow-plane kernel
         const bool narrow = G == 1 && wmx <= 64;
         const int32_t nt_req = h->opts.band_threads == 32 && !narrow ? 0 : h->opts.band_threads;
         hs.band_nt = nt_req ? nt_req : narrow ? 32 : (nparts * G > nsm ? 256 : 512);

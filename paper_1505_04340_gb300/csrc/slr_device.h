@@ -67,6 +67,7 @@ template <typename T>
 struct DevOperator {
     BandBlock* band = nullptr;     // [p]
     T* bfac = nullptr;
+    int64_t bfac_len = 0;          // its elements
     int32_t band_G = 1;            // CTAs per subdomain (thread-block cluster size)
     int32_t band_nbuf = 0;         // ring slots of the band solve (0: the default count)
     int32_t band_nt = 512;         // threads per band-solve CTA: 512 (one per SM) or 256 (two per SM)
@@ -176,9 +177,9 @@ std::vector<BandTcBlock> band_tc_layout(const std::vector<BandBlock>& run_order,
 cudaError_t launch_band_tc_pack(int32_t mma_dtype, const BandTcBlock* band, int32_t p, int32_t cmax,
                                 const double* scr, const int64_t* soff, unsigned char* fac, bool indef,
                                 cudaStream_t st);
-// K1 with one warp per subdomain, for planes of at most 64 rows packed as one slice (slr_band_warp.cu)
+// K1 for planes of at most 64 rows packed as one slice: a CTA of four warps per subdomain (slr_band_narrow.cu)
 template <typename T>
-cudaError_t launch_band_warp(const DevOperator<T>& op, int32_t p, const T* in, int64_t ldi, T* out, int64_t ldo,
+cudaError_t launch_band_narrow(const DevOperator<T>& op, int32_t p, int32_t wmax, const T* in, int64_t ldi, T* out, int64_t ldo,
                              const T* base, int64_t ldb, int32_t nrhs, cudaStream_t st);
 cudaError_t launch_band_solve_tc(const DevOperator<float>& op, int32_t p, const float* in, int64_t ldi, float* out,
                                  int64_t ldo, const float* base, int64_t ldb, int32_t nrhs, cudaStream_t st);
