@@ -245,7 +245,6 @@ k_band_tc(const BandTcBlock* __restrict__ blocks, const unsigned char* __restric
     const int nU = b.nU, nL = b.nL;
     const int nblk = 4 * c - 2;
     auto tiles_of = [&](int type) { return (type == 0 || type == 3) ? nU : nL; };
-    auto fills_of = [&](int type) { return (tiles_of(type) + stiles - 1) / stiles; };
     auto fail = [&]() {
         atomicExch(err, 1);
         *abort_flag = 1;
@@ -253,15 +252,15 @@ k_band_tc(const BandTcBlock* __restrict__ blocks, const unsigned char* __restric
 
     if (tid == 0) {
         // ---------------------------------------------------------------- producer
-        int f = 0;
+        int f = 0, s = 0;                               // copies issued, slot of the next one
+        uint32_t par = 1;                               // parity of the slot's last release
         for (int q = 0; q < nblk && !*abort_flag; ++q) {
             const BtBlock bk = bt_block(q, c);
             const int nt = tiles_of(bk.type);
             const int64_t boff = bk.type == 0 ? 0 : bk.type == 1 ? nU : bk.type == 2 ? nU + nL : nU + 2 * nL;
             const unsigned char* src = fac + b.foff + ((int64_t)bk.plane * (2 * nU + 2 * nL) + boff) * kSub;
             for (int t0 = 0; t0 < nt; t0 += stiles, ++f) {
-                const int s = f % nslot;
-                if (f >= nslot && !tc::mbar_wait(&empty[s], (uint32_t)(((f / nslot) - 1) & 1), kBtSpin)) {
+                if (f >= nslot && !tc::mbar_wait(&empty[s], par, kBtSpin)) {
                     fail();
                     break;
                 }
@@ -275,6 +274,10 @@ k_band_tc(const BandTcBlock* __restrict__ blocks, const unsigned char* __restric
                         tc::smem_addr(ring + (size_t)s * stiles * kSub)),
                     "l"(src + (int64_t)t0 * kSub), "r"(bytes), "r"(tc::smem_addr(&full[s]))
                     : "memory");
+                if (++s == nslot) {
+                    s = 0;
+                    par ^= 1;
+                }
             }
         }
         // no copy of this CTA still writes its shared memory when it leaves: the last
@@ -285,34 +288,55 @@ k_band_tc(const BandTcBlock* __restrict__ blocks, const unsigned char* __restric
         }
     } else if (tid == 32) {
         // ---------------------------------------------------------------- MMA issuer
+        // One thread issues every MMA, so its instructions are the block's critical path:
+        // the slot, its parity and both descriptors are carried along instead of being
+        // formed anew for each sub-tile (with two divisions and a modulo per sub-tile an
+        // MMA took 540 cycles to issue, 24,000 of a block's 28,000; the MMA itself takes about 20).
         const uint32_t idesc = tc::instr_desc(AB, 128, NP);
-        int f = 0;
+        const uint64_t ring_desc = tc::smem_desc(tc::smem_addr(ring), 128, 256);
+        const uint64_t vec_desc = tc::smem_desc(tc::smem_addr(vbuf), 128, sbo_v);
+        constexpr uint64_t kSubDesc = kSub >> 4, kStepDesc = 256 >> 4;   // one sub-tile, one K-step (16-byte units)
+        int s = 0;                                      // slot and parity of the copy in use
+        uint32_t par = 0;
         for (int q = 0; q < nblk; ++q) {
+            const BtBlock bk = bt_block(q, c);
+            const bool upper = bk.type == 0 || bk.type == 3;
             if (!tc::mbar_wait(opnd_bar, (uint32_t)(q & 1), kBtSpin)) fail();
             if (*abort_flag) break;
             tc::fence_after_sync();
-            const BtBlock bk = bt_block(q, c);
-            const bool upper = bk.type == 0 || bk.type == 3;
             // the operand: t (D blocks) or Y / X (O blocks), written by the last epilogue
-            const uint32_t vb = tc::smem_addr(vbuf);
-            int t = 0;
+            int left = tiles_of(bk.type), in_slot = 0;  // sub-tiles of the block, of the slot
+            uint64_t ad = 0;
             bool ok = true;
-            for (int mt = 0; mt < nM && ok; ++mt)
-                for (int ks = bt_k0(upper, mt, KS); ks < bt_k1(upper, mt, W, KS); ++ks, ++t) {
-                    const int fl = f + t / stiles, s = fl % nslot, in_slot = t % stiles;
-                    if (in_slot == 0 && !tc::mbar_wait(&full[s], (uint32_t)((fl / nslot) & 1), kBtSpin)) {
-                        fail();
-                        ok = false;
-                        break;
+            for (int mt = 0; mt < nM && ok; ++mt) {
+                const int k0 = bt_k0(upper, mt, KS), k1 = bt_k1(upper, mt, W, KS);
+                const uint32_t d = tmem + (uint32_t)(mt * CS);
+                uint64_t bd = vec_desc + kStepDesc * k0;
+                for (int ks = k0; ks < k1; ++ks) {
+                    if (in_slot == 0) {
+                        if (!tc::mbar_wait(&full[s], par, kBtSpin)) {
+                            fail();
+                            ok = false;
+                            break;
+                        }
+                        ad = ring_desc + kSubDesc * (uint32_t)(s * stiles);
                     }
-                    const uint32_t sa = tc::smem_addr(ring + ((size_t)s * stiles + in_slot) * kSub);
-                    tc::mma<AB>(tmem + (uint32_t)(mt * CS), tc::smem_desc(sa, 128, 256),
-                                tc::smem_desc(vb + 256u * ks, 128, sbo_v), idesc, ks > bt_k0(upper, mt, KS));
-                    const bool last_of_fill = in_slot == stiles - 1 || t == tiles_of(bk.type) - 1;
-                    if (last_of_fill) tc::commit(&empty[s]);
+                    tc::mma<AB>(d, ad, bd, idesc, ks > k0);
+                    ad += kSubDesc;
+                    bd += kStepDesc;
+                    ++in_slot;
+                    --left;
+                    if (in_slot == stiles || left == 0) {       // the slot's last sub-tile
+                        tc::commit(&empty[s]);
+                        in_slot = 0;
+                        if (++s == nslot) {
+                            s = 0;
+                            par ^= 1;
+                        }
+                    }
                 }
+            }
             if (!ok) break;
-            f += fills_of(bk.type);
             tc::commit(acc_bar);
         }
         tc::commit(fin_bar);                            // every MMA issued has completed
