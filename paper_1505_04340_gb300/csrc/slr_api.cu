@@ -961,11 +961,18 @@ slr_status setup_impl(slr_handle h, int32_t n, const int32_t* rowptr, const int3
         const int32_t req = h->opts.band_split;        // 0 = automatic
         if (req == 1 || req == 2 || req == 4) {
             if (band_split_ok(wmx, req)) G = req;
-        } else if (G == 1 && 2 * nparts <= nsm && wmx >= 64) {
-            // a subdomain's planes are a dependent chain: with few subdomains two
-            // CTAs (a cluster) per subdomain put twice the SMs on it (measured
-            // faster in both precisions on 16^3 boxes; four CTAs need two waves)
-            G = 2;
+        } else if (G == 1) {
+            // A subdomain's planes are a dependent chain, so few subdomains are split over
+            // a cluster.  FP64 is bound by its pipe and takes every SM it can get: planes
+            // of 128 rows or more go four ways (two ways) while two 256-thread CTAs per SM
+            // hold all slices, so that one slice's exchange hides behind the other's
+            // products (W = 225, one column, CTAs per subdomain 1, 2, 4: 64 subdomains 564, 361,
+            // 327 us, 27: 563, 359, 240, 8: 421, 274, 223; W = 196, 125 subdomains: 422, 379, 422; W = 100, 64
+            // subdomains: 162, 124, 136).  FP32 takes two while each slice has an SM of its
+            // own, four if those have (64 subdomains 143, 102, 168 us; 27: 142, 99, 93; 8: 112, 89, 86).
+            const bool fp64 = h->opts.precision == SLR_PREC_FP64;
+            if (wmx >= 128 && 4 * nparts <= (fp64 ? 2 * nsm : nsm)) G = 4;
+            else if ((wmx >= 64 && 2 * nparts <= nsm) || (fp64 && wmx >= 128 && nparts <= nsm)) G = 2;
         }
         // Section 5.2: factor the B_i on the device when every plane fits its kernel (at
         // most 256 rows), else on the host

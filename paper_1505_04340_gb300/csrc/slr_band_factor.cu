@@ -298,21 +298,21 @@ k_band_pack(const BandBlock* __restrict__ band, int32_t cmax, int32_t G, const d
     for (int rb = 0; rb < b.nrb[g]; ++rb) {
         const int R0 = 32 * b.rbmap[g][rb];
         const int cu0 = min(W, R0), cl1 = min(W, min(R0 + 31, W - 1) + 1);
-        const int nu = W - cu0;
+        const int nu = (W - cu0 + 3) & ~3, nl = (cl1 + 3) & ~3;     // whole quads
         for (int e = threadIdx.x; e < 32 * nu; e += blockDim.x) {   // upper: rows r <= cc
-            const int cc = cu0 + e / 32, r = R0 + (e & 31), l = J * W + r;
-            const bool in = r < W && r <= cc;
+            const int cc = cu0 + 4 * (e / 128) + (e & 3), r = R0 + (e & 127) / 4, l = J * W + r;
+            const bool in = r < W && r <= cc && cc < W;
             Uf[(su * 32) + e] = in && J > 0 && l < m ? (T)(O[(int64_t)r * W + cc] * sgn(J - 1, cc)) : T(0);
             Ub[(su * 32) + e] = in ? (T)X[(int64_t)cc * W + r] : T(0);
         }
-        for (int e = threadIdx.x; e < 32 * cl1; e += blockDim.x) {  // lower: rows r >= cc
-            const int cc = e / 32, r = R0 + (e & 31), lc = J * W + cc;
-            const bool in = r < W && r >= cc;
+        for (int e = threadIdx.x; e < 32 * nl; e += blockDim.x) {   // lower: rows r >= cc
+            const int cc = 4 * (e / 128) + (e & 3), r = R0 + (e & 127) / 4, lc = J * W + cc;
+            const bool in = r < W && r >= cc && cc < W;
             Lf[(sl * 32) + e] = in ? (T)(X[(int64_t)r * W + cc] * sgn(J, r)) : T(0);
             Lb[(sl * 32) + e] = in && J > 0 && lc < m ? (T)O[(int64_t)cc * W + r] : T(0);
         }
         su += nu;
-        sl += cl1;
+        sl += nl;
     }
 }
 

@@ -8,6 +8,7 @@
 #include <atomic>
 #include <cstdint>
 #include <mutex>
+#include <type_traits>
 
 #include "slr_device.h"
 
@@ -17,11 +18,10 @@ namespace slr {
 
 namespace {
 
-constexpr int kMaxBuf = 8;         // ring slots at most
-constexpr int kMinBuf = 2;         // ring slots at least
-constexpr int kDefBuf = 2;         // ring slots unless the operator asks for another count
-                                   // (two large slots measured fastest: per-chunk latency dominates)
-constexpr int kMinSlot = 16 * 1024;   // bytes per ring slot at least
+constexpr int kMaxBuf = 8;         // ring slots of a warp at most
+constexpr int kMinBuf = 2;         // ring slots of a warp at least
+constexpr int kDefBuf = 2;         // unless the operator asks for another count
+constexpr int kMaxCq = 16;         // quads per slot at most
 // Shared memory a CTA may use: the opt-in maximum for 512-thread CTAs (one per
 // SM); for 256-thread CTAs, half an SM's 228 KB less its per-CTA reserve, so
 // two CTAs (two subdomains) share each SM.
@@ -129,18 +129,6 @@ __device__ __forceinline__ void cluster_barrier() {
     }
 }
 
-// Column c of every block goes to warp c mod KW whatever the chunk boundaries,
-// so each warp's partial sums, and the result, do not depend on the ring's
-// slot size (which varies with the right-hand sides per CTA).
-template <int KW>
-__device__ __forceinline__ int first_col(int lo, int warp) { return lo + ((warp - lo % KW) + KW) % KW; }
-
-struct Geom {
-    int W, c, g;
-    int nU, nL;
-    int64_t base, PS, SU, SL;
-};
-
 // Block types: 0 O_J (upper, fwd), 1 D_J (lower, fwd), 2 O_J^T (lower, bwd), 3 D_J^T (upper, bwd).
 // Stream order: forward D_0, (O_J, D_J) J = 1..c-1; backward D_{c-1}^T, then
 // (O_{J+1}^T, D_J^T) J = c-2..0 (O_{J+1}^T is stored with plane J+1).
@@ -154,169 +142,185 @@ __device__ __forceinline__ void next_block(int c, int& type, int& plane) {
     }
 }
 
-__device__ __forceinline__ int64_t block_off(const Geom& q, int type) {
-    return type == 0 ? 0 : type == 1 ? q.SU : type == 2 ? q.SU + q.SL : q.SU + 2 * q.SL;
+// bytes of the barriers and tables at the start of a CTA's shared memory
+__host__ __device__ inline int band_head_bytes(int nt) {
+    return (nt / 32 * kMaxBuf * 8 + 4 * 8 + kRB * 4 + 2 * kRB * 8 + 127) / 128 * 128;
+}
+
+// N consecutive values from shared memory, as wide as they allow (p aligned to
+// min(16, N sizeof(T)) bytes)
+template <typename T, int N>
+__device__ __forceinline__ void ld_vec(const T* p, T (&v)[N]) {
+    if constexpr (sizeof(T) == 4 && N % 4 == 0) {
+#pragma unroll
+        for (int q = 0; q < N; q += 4) {
+            const float4 a = *reinterpret_cast<const float4*>(p + q);
+            v[q] = a.x; v[q + 1] = a.y; v[q + 2] = a.z; v[q + 3] = a.w;
+        }
+    } else if constexpr (sizeof(T) == 8 && N % 2 == 0) {
+#pragma unroll
+        for (int q = 0; q < N; q += 2) {
+            const double2 a = *reinterpret_cast<const double2*>(p + q);
+            v[q] = a.x; v[q + 1] = a.y;
+        }
+    } else {
+#pragma unroll
+        for (int q = 0; q < N; ++q) v[q] = p[q];
+    }
 }
 
 }  // namespace
 
-// NT threads per CTA: 512 (one CTA per SM, 4 warps per SM sub-partition to hide
-// the load->FMA latency) or 256 (two CTAs, two subdomains, per SM).
+// NT threads per CTA: 512 (one CTA per SM, 4 warps per SM sub-partition) or 256
+// (two CTAs, two subdomains, per SM).  nr <= NR right-hand sides.
+//
+// What bounds it is the chain of 4 c - 2 blocks (c planes); per block the slice's
+// bytes, FP64's multiply-adds (its pipe takes a warp's in about 17 cycles) and
+// the fixed cost of a step: products, one CTA barrier, the rows' sums, the exchange.
+// So a warp's part of a block is a plain run over its quads, with a branch only where
+// its row block changes.
 template <typename T, int NR, int G, int NT>
 __global__ void __launch_bounds__(NT, 512 / NT)
-k_band_solve2(const BandBlock* __restrict__ blocks, const T* __restrict__ fac, const T* in, int64_t ldi, T* out,
-              int64_t ldo, const T* base, int64_t ldb, int32_t* err, int nbuf, int slot) {
-    constexpr int kT = NT;         // threads per CTA
-    constexpr int kW = NT / 32;    // warps per CTA
+k_band_wide(const BandBlock* __restrict__ blocks, const T* __restrict__ fac, const T* in, int64_t ldi, T* out,
+            int64_t ldo, const T* base, int64_t ldb, int32_t* err, int nr, int nbuf, int cq, int once) {
+    constexpr int kW = NT / 32;                           // warps per CTA
+    constexpr int NIT = (kRB * NR + kW - 1) / kW;         // (row block, right-hand side) pairs a warp owns
     extern __shared__ __align__(128) unsigned char smem[];
     const int sub = blockIdx.x / G;
     const int g = (G > 1) ? (int)cg::this_cluster().block_rank() : 0;
-    const BandBlock b = blocks[sub];
-    if (b.m == 0) return;                       // uniform across the cluster
-    const int W = b.w, c = b.c, m = b.m;
+    const BandBlock& b = blocks[sub];
+    const int W = b.w, c = b.c, m = b.m, WP = (W + 3) & ~3;
+    if (m == 0) return;                         // uniform across the cluster
+    const int SU = b.SU, SL = b.SL, row0 = b.row0, nrb = b.nrb[g];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
-    // ---- shared memory carve-up: barriers, tables and vectors, then the ring
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem);              // [kMaxBuf]
-    uint64_t* empty = full + kMaxBuf;                                 // [kMaxBuf]
-    uint64_t* vbar = empty + kMaxBuf;                                 // [3] t (two buffers), y/x
-    int* segU = reinterpret_cast<int*>(vbar + 4);                    // [kRB+1] first segment of row block rb
-    int* segL = segU + (kRB + 1);                                    // [kRB+1]
-    int* hdr = segL + (kRB + 1);                                     // nU, nL, segments per chunk, abort
-    uintptr_t vp = reinterpret_cast<uintptr_t>(hdr + 4);
-    vp = (vp + 15) & ~uintptr_t(15);
-    T* vst = reinterpret_cast<T*>(vp);              // [NR][W] y_{J-1} (fwd) / x_{J+1} (bwd), whole plane
-    T* vt = vst + NR * W;                           // [2][NR][W] t, whole plane, by phase parity
-    T* part = vt + 2 * NR * W;                      // [kW][NR][256] per-warp partial sums
-    uintptr_t rp = reinterpret_cast<uintptr_t>(part + kW * NR * 256);
-    unsigned char* ring = reinterpret_cast<unsigned char*>((rp + 127) & ~uintptr_t(127));   // nbuf x slot bytes
+    // ---- shared memory carve-up: barriers, tables and vectors, then the rings
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem) + warp * kMaxBuf;   // [kW][kMaxBuf]
+    uint64_t* vbar = reinterpret_cast<uint64_t*>(smem) + kW * kMaxBuf;      // [3] t (two buffers), y/x
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(vbar + 3);
+    int* R0s = reinterpret_cast<int*>(vbar + 4);                            // [kRB] first row of each row block
+    int2* pw = reinterpret_cast<int2*>(R0s + kRB);                          // [2][kRB] first and last warp of a row
+                                                                            // block (upper, lower)
+    T* vst = reinterpret_cast<T*>(smem + band_head_bytes(NT));              // [WP][NR] y_{J-1} / x_{J+1}, whole plane
+    T* vt = vst + NR * WP;                          // [2][WP][NR] t, whole plane, by phase parity
+    T* part = vt + 2 * NR * WP;                     // [kW + kRB][NR][32] pieces
+    const int slot = cq * 128;                      // elements
+    uintptr_t rp = (reinterpret_cast<uintptr_t>(part + (kW + kRB) * NR * 32) + 127) & ~uintptr_t(127);
+    T* ring = reinterpret_cast<T*>(rp) + (size_t)warp * nbuf * slot;
 
-    Geom q;
-    q.W = W;
-    q.c = c;
-    q.g = g;
-    q.SU = b.SU;
-    q.SL = b.SL;
-    q.PS = (int64_t)G * 2 * (b.SU + b.SL);
-    q.base = b.foff + (int64_t)g * 2 * (b.SU + b.SL);
-
-    // this slice's row blocks: first plane row of each (past W: none)
-    const int nrb = b.nrb[g];
-    int R0[kRB];
-#pragma unroll
-    for (int rb = 0; rb < kRB; ++rb) R0[rb] = rb < nrb ? 32 * b.rbmap[g][rb] : W;
+    const int64_t PS = (int64_t)G * 2 * (SU + SL);
+    const T* facg = fac + b.foff + (int64_t)g * 2 * (SU + SL);
     // Every row of a plane has one owner in the cluster.  A phase of a vector
-    // barrier completes with 1 + nrb arrivals (thread 0 arming it, and each of
-    // this slice's owner warps once its rows are stored here) and the bytes of
-    // the other slices' rows, stored by their owners with st.async.
+    // barrier completes with 1 + narr arrivals (thread 0 arming it, and each warp
+    // that owns rows once they are stored here) and the bytes of the other
+    // slices' rows, stored by their owners with st.async.
     int my_rows = 0;
+    for (int rb = 0; rb < nrb; ++rb) my_rows += min(32, W - 32 * b.rbmap[g][rb]);
+    const uint32_t rbytes = (uint32_t)((W - my_rows) * nr * (int)sizeof(T));
+    const int narr = min(kW, nrb * nr);
+
+    // this warp's share of an upper (0) and a lower (1) block: first quad of the slice's
+    // block, quads, and the first quad's row block and column
+    int sq0[2], snq[2], srb[2], scol[2];
 #pragma unroll
-    for (int rb = 0; rb < kRB; ++rb)
-        if (rb < nrb) my_rows += min(32, W - R0[rb]);
-    const uint32_t rbytes = (uint32_t)((W - my_rows) * NR * (int)sizeof(T));
-    if (tid == 0) {
-        int a = 0, d = 0;
-        for (int rb = 0; rb <= kRB; ++rb) {
-            segU[rb] = a;
-            segL[rb] = d;
-            if (rb < nrb) {
-                a += W - seg_cU0(W, R0[rb]);
-                d += seg_cL1(W, R0[rb]);
+    for (int t = 0; t < 2; ++t) {
+        auto quads = [&](int rb) {
+            const int r0 = 32 * b.rbmap[g][rb];
+            return ((t == 0 ? W - seg_cU0(W, r0) : seg_cL1(W, r0)) + 3) >> 2;
+        };
+        int Q = 0;
+        for (int rb = 0; rb < nrb; ++rb) Q += quads(rb);
+        // (with fewer quads than warps, one each: every share before the last is non-empty)
+        const int ew = min(kW, Q);
+        sq0[t] = warp < ew ? Q * warp / ew : Q;
+        snq[t] = warp < ew ? Q * (warp + 1) / ew - sq0[t] : 0;
+        srb[t] = scol[t] = 0;
+        int q = 0;
+        for (int rb = 0; rb < nrb; ++rb) {
+            const int n = quads(rb);
+            if (tid == 0) pw[t * kRB + rb] = make_int2(((q + 1) * ew - 1) / Q, ((q + n) * ew - 1) / Q);
+            if (sq0[t] >= q && sq0[t] < q + n) {
+                srb[t] = rb;
+                scol[t] = 4 * (sq0[t] - q) + (t == 0 ? seg_cU0(W, 32 * b.rbmap[g][rb]) : 0);
             }
+            q += n;
         }
-        const int per = max(1, slot / (32 * (int)sizeof(T)));   // whole segments per chunk
-        hdr[0] = (a + per - 1) / per;
-        hdr[1] = (d + per - 1) / per;
-        hdr[2] = per;
-        hdr[3] = 0;                                // set once a bounded wait of this CTA expires
-        for (int i = 0; i < nbuf; ++i) {
-            mbar_init(&full[i], 1);
-            mbar_init(&empty[i], kW);
-        }
-        for (int i = 0; i < 3; ++i) mbar_init(&vbar[i], 1 + nrb);
+    }
+    if (tid < nrb) R0s[tid] = 32 * b.rbmap[g][tid];
+    if (lane == 0)
+        for (int i = 0; i < nbuf; ++i) mbar_init(&full[i], 1);
+    if (tid == 0) {
+        *abort_flag = 0;                                  // set once a bounded wait of this CTA expires
+        for (int i = 0; i < 3; ++i) mbar_init(&vbar[i], 1 + narr);
         for (int i = 0; i < 3; ++i) {
             if (rbytes) mbar_arrive_expect_tx(&vbar[i], rbytes);
             else mbar_arrive(&vbar[i]);
         }
-        fence_mbar_init();
     }
+    if (lane == 0) fence_mbar_init();
+    // the vectors' entries past W and past nr stay zero
+    for (int i = tid; i < 3 * NR * WP; i += NT) vst[i] = T(0);
     __syncthreads();
-    q.nU = hdr[0];
-    q.nL = hdr[1];
-    const int per = hdr[2];
-    // forward: D_0 (lower), then (O_J upper, D_J lower); backward: D_{c-1}^T (upper), then (O^T lower, D^T upper)
-    const int total = q.nL + q.nU + 2 * (c - 1) * (q.nU + q.nL);
 
-    // first and one-past-last element of chunk ix of a block: segments [ix per, ...)
-    auto chunk_src = [&](int type, int plane, int ix, int64_t& e0, int64_t& e1) {
-        const bool up = (type == 0 || type == 3);
-        const int nseg = up ? segU[kRB] : segL[kRB];
-        e0 = q.base + (int64_t)plane * q.PS + block_off(q, type) + (int64_t)ix * per * 32;
-        e1 = e0 + (int64_t)(min(per, nseg - ix * per)) * 32;
-    };
-    // thread 0 issues chunks in stream order; its cursor is the next chunk to issue
-    int cur_type = 1, cur_plane = 0, cur_ix = 0, issued = 0;
+    // lane 0 of a warp issues the copies of its share in stream order, cq quads at most each
+    int itype = 1, iplane = 0, iq = 0, issued = 0, islot = 0;   // next copy: block, first quad; its slot
+    const uint64_t pol = policy_stream(once != 0);
     auto issue_next = [&]() {
-        if (cur_plane < 0) return;                 // past the end of the stream: nothing to copy
-        int64_t e0, e1;
-        chunk_src(cur_type, cur_plane, cur_ix, e0, e1);
-        // whole segments of 32 values: start and size are multiples of 128 bytes
-        const uint32_t bytes = (uint32_t)((e1 - e0) * (int64_t)sizeof(T));
-        const int sl = issued % nbuf;
-        uint64_t* bar = &full[sl];
-        mbar_arrive_expect_tx(bar, bytes);
-        bulk_g2s(ring + (size_t)sl * slot, fac + e0, bytes, bar);
+        // (a warp may have a share of one block type only)
+        while (iplane >= 0 && ((itype == 0 || itype == 3) ? snq[0] : snq[1]) == 0) next_block(c, itype, iplane);
+        if (iplane < 0) return;
+        const bool up = itype == 0 || itype == 3;
+        const int n = min(cq, (up ? snq[0] : snq[1]) - iq);
+        const int64_t off = (int64_t)iplane * PS +
+                            (itype == 0 ? 0 : itype == 1 ? SU : itype == 2 ? SU + SL : SU + 2 * SL);
+        const uint32_t bytes = (uint32_t)(n * 128 * (int)sizeof(T));
+        mbar_arrive_expect_tx(&full[islot], bytes);
+        bulk_g2s_pol(ring + (size_t)islot * slot, facg + off + ((up ? sq0[0] : sq0[1]) + iq) * 128, bytes,
+                     &full[islot], pol);
         ++issued;
-        const int nch = (cur_type == 0 || cur_type == 3) ? q.nU : q.nL;
-        if (++cur_ix == nch) {
-            cur_ix = 0;
-            next_block(c, cur_type, cur_plane);
+        iq += n;
+        if (iq == (up ? snq[0] : snq[1])) {
+            iq = 0;
+            next_block(c, itype, iplane);
         }
+        if (++islot == nbuf) islot = 0;
     };
     // After a bounded wait expires the CTA aborts: the status word and the
-    // CTA's abort flag (hdr[3]) are set, no further copy is issued, the block
-    // products and the vector waits are skipped, and before it exits thread 0
-    // waits for the copies it issued.
-    volatile int* abort_flag = hdr + 3;
-    auto wait_bar = [&](uint64_t* bar, uint32_t par) -> bool {
+    // CTA's abort flag are set, no further copy is issued, and before it exits each
+    // warp waits for the copies it issued.  The CTA goes through the rest of its steps
+    // with whatever its buffers hold (no wait is taken again).
+    auto fail = [&]() {
+        atomicExch(err, 1);
+        *abort_flag = 1;
+    };
+    int kslot = 0;                                        // slot and parity of the next copy to read
+    uint32_t kpar = 0;
+    auto wait_full = [&]() {
         long long it = 0;
-        while (!mbar_try_wait(bar, par)) {
-            if (++it > kSpin) {
-                atomicExch(err, 1);
-                *abort_flag = 1;
-                return false;
+        while (!mbar_try_wait(&full[kslot], kpar)) {
+            if (++it > kSpin || *abort_flag) {
+                fail();
+                break;
             }
         }
-        return true;
-    };
-    // chunk k's data has landed (the (k / nbuf)-th fill of its slot); false once the CTA
-    // aborted.  The answer is the same for the whole warp (all lanes saw the data land).
-    auto wait_full = [&](int k) -> bool {
-        bool ok = !*abort_flag && wait_bar(&full[k % nbuf], (uint32_t)((k / nbuf) & 1));
-        return __all_sync(0xffffffffu, ok);
-    };
-    // this warp is done with chunk k's slot (its release is ordered after a store
-    // of the abort flag, so the refilling thread sees the flag once it has the slot)
-    auto release = [&](int k) {
         __syncwarp();
-        if (lane == 0) mbar_arrive(&empty[k % nbuf]);
     };
-    // thread 0, before consuming chunk k: once every warp has released chunk
-    // k - 1, its slot takes the next chunk of the stream (unless the CTA aborted:
-    // a warp whose wait for chunk k - 1 expired may have left that copy in flight)
-    auto refill = [&](int k) {
-        if (tid == 0 && k >= 1 && issued < total && !*abort_flag) {
-            if (wait_bar(&empty[(k - 1) % nbuf], (uint32_t)(((k - 1) / nbuf) & 1)) && !*abort_flag) {
-                fence_proxy_async();
-                issue_next();
-            }
+    // the warp has read its slot: lane 0 refills it (nothing is issued after an abort: a
+    // copy whose wait expired may still be in flight)
+    auto next_slot = [&]() {
+        __syncwarp();
+        if (lane == 0 && iplane >= 0 && !*abort_flag) {
+            fence_proxy_async();
+            issue_next();
+        }
+        if (++kslot == nbuf) {
+            kslot = 0;
+            kpar ^= 1;
         }
     };
-    // thread 0 at exit after an abort: the last copy issued into each slot has
-    // landed (the fills of a slot are issued one after another, each once the
-    // previous one was consumed, so the last one completing means all did)
+    // at exit after an abort: the last copy issued into each slot has landed
     auto drain = [&]() {
-        if (tid != 0 || !*abort_flag) return;
+        if (lane != 0 || !*abort_flag) return;
         for (int sl = 0; sl < nbuf && sl < issued; ++sl) {
             const int last = sl + ((issued - 1 - sl) / nbuf) * nbuf;
             long long it = 0;
@@ -336,37 +340,33 @@ k_band_solve2(const BandBlock* __restrict__ blocks, const T* __restrict__ fac, c
     // pass's last t and the backward pass's first t have no exchange of y
     // between them, so a fast peer can send the second before a slow CTA has
     // read the first.  y/x needs one buffer (an exchange of t always lies between
-    // two of its phases).  A wait that expires sets the abort flag; the barrier
-    // is then left un-armed (thread 0 never arrives twice in one phase).
-    auto wait_vec = [&](uint64_t* bar, uint32_t par) -> bool {
-        bool ok = false;
-        if (!*abort_flag) {
-            long long it = 0;
-            ok = true;
-            while (!mbar_try_wait_cluster(bar, par)) {
-                if (++it > kSpin) {
-                    atomicExch(err, 1);
-                    *abort_flag = 1;
-                    ok = false;
-                    break;
-                }
-            }
-            if (ok && tid == 0) {
-                if (rbytes) mbar_arrive_expect_tx(bar, rbytes);
-                else mbar_arrive(bar);
+    // two of its phases).  After a wait that expired the barrier
+    // is left un-armed (thread 0 never arrives twice in one phase).
+    auto wait_vec = [&](uint64_t* bar, uint32_t par) {
+        long long it = 0;
+        bool ok = true;
+        while (!mbar_try_wait_cluster(bar, par)) {
+            if (++it > kSpin || *abort_flag) {
+                fail();
+                ok = false;
+                break;
             }
         }
-        return __all_sync(0xffffffffu, ok);
+        if (ok && tid == 0) {
+            if (rbytes) mbar_arrive_expect_tx(bar, rbytes);
+            else mbar_arrive(bar);
+        }
+        __syncwarp();
     };
-    // owner rows of a phase into vector vec (element j W + own_r) of every CTA.
+    // entry (r, j) of a phase's vector vec into every CTA.
     // An aborted CTA sends nothing more: its peers' waits for its rows then
     // expire and they abort in turn, so at most a phase or two of bytes reach a
     // barrier this CTA no longer arms.
     auto send = [&](T* vec, uint64_t* bar, int j, int r, T v) {
-        if (*abort_flag) return;
-        vec[j * W + r] = v;
+        vec[r * NR + j] = v;
         if constexpr (G > 1) {
-            const uint32_t a = smem_u32(vec + j * W + r), mb = smem_u32(bar);
+            if (*abort_flag) return;
+            const uint32_t a = smem_u32(vec + r * NR + j), mb = smem_u32(bar);
 #pragma unroll
             for (int pr = 0; pr < G; ++pr)
                 if (pr != g) st_async(peer_addr(a, pr), v, peer_addr(mb, pr));
@@ -374,182 +374,209 @@ k_band_solve2(const BandBlock* __restrict__ blocks, const T* __restrict__ fac, c
     };
     // an owner warp, once all its rows of a phase are stored here (all of its lanes)
     auto arrive_local = [&](uint64_t* bar) {
-        if (warp < nrb) {
+        if (warp < narr) {
             __syncwarp();
             if (lane == 0 && !*abort_flag) mbar_arrive(bar);
         }
     };
 
-    if (tid == 0)
-        while (issued < nbuf && issued < total) issue_next();
+    if (lane == 0)
+        while (issued < nbuf && iplane >= 0) issue_next();
     // every CTA of the cluster has armed its barriers before any st.async reaches it
     cluster_barrier<G>();
 
-    int k = 0;
-    T acc[kRB][NR];
-    // acc[rb][j] = sum over the block's segments of row block rb of seg[lane] * vin[j][column];
-    // vin is complete once phase `par` of vector barrier `vb` has
-    auto run_block = [&](int type, int plane, const T* vin, uint64_t* vb, uint32_t par) {
-        const bool upper = (type == 0 || type == 3);
+    // One block: this warp's share times the vector vin (complete once phase `par` of
+    // vector barrier `vb` has), its pieces to `part`.
+    auto run_block = [&](auto up, const T* vin, uint64_t* vb, uint32_t par) {
+        constexpr bool UP = decltype(up)::value;
+        constexpr int ST = UP ? 0 : 1;
+        int n = snq[ST], rb = srb[ST], col = scol[ST];
+        wait_vec(vb, par);
+        T acc[NR], ac2[NR];
 #pragma unroll
-        for (int rb = 0; rb < kRB; ++rb)
-#pragma unroll
-            for (int j = 0; j < NR; ++j) acc[rb][j] = T(0);
-        const int nch = upper ? q.nU : q.nL;
-        const int* seg = upper ? segU : segL;
-        bool vok = true, waited = false;
-        for (int ix = 0; ix < nch; ++ix, ++k) {
-            refill(k);
-            const bool landed = wait_full(k);
-            if (!waited) {                 // the input vector (after the block's first data)
-                vok = wait_vec(vb, par);
-                waited = true;
-            }
-            if (!landed || !vok) {         // aborted: no product
-                release(k);
-                continue;
-            }
-            const int s0 = ix * per, s1 = min(s0 + per, seg[kRB]);
-            const T* P = reinterpret_cast<const T*>(ring + (size_t)(k % nbuf) * slot);
-#pragma unroll
-            for (int rb = 0; rb < kRB; ++rb) {
-                if (rb >= nrb) break;
-                const int sa = max(s0, seg[rb]), sb = min(s1, seg[rb + 1]);
-                if (sa >= sb) continue;
-                const int cb0 = upper ? seg_cU0(W, R0[rb]) : 0;         // column of segment seg[rb]
-                const int ca = cb0 + (sa - seg[rb]), ce = cb0 + (sb - seg[rb]);
-                int cc = first_col<kW>(ca, warp);
-                const T* Ps = P + (sa - s0 + (cc - ca)) * 32 + lane;
+        for (int j = 0; j < NR; ++j) acc[j] = ac2[j] = T(0);
+        int left = n > 0 ? ((UP ? W : seg_cL1(W, R0s[rb])) - col + 3) >> 2 : 0;   // quads of the row block
+        const T* V = vin + col * NR;
+        while (n > 0) {
+            wait_full();
+            const T* P = ring + (size_t)kslot * slot + lane * 4;
+            int nc = min(cq, n);
+            n -= nc;
+            while (true) {
+                const int t = min(nc, left);
 #pragma unroll 2
-                for (; cc < ce; cc += kW, Ps += kW * 32) {
-                    const T a = *Ps;
+                for (int i = 0; i < t; ++i) {
+                    T a[4];
+                    ld_vec<T, 4>(P, a);
+                    // two chains per right-hand side: even and odd columns
+                    constexpr int U = NR < 4 ? 4 / NR : 1;   // columns per load of the vector
 #pragma unroll
-                    for (int j = 0; j < NR; ++j) acc[rb][j] = fma(a, vin[j * W + cc], acc[rb][j]);
+                    for (int u = 0; u < 4; u += U) {
+                        T v[U * NR];
+                        ld_vec<T, U * NR>(V + u * NR, v);
+#pragma unroll
+                        for (int w = 0; w < U; ++w)
+#pragma unroll
+                            for (int j = 0; j < NR; ++j)
+                                if (NR <= 2 || j < nr) {
+                                    T& s = ((u + w) & 1) ? ac2[j] : acc[j];
+                                    s = fma(a[u + w], v[w * NR + j], s);
+                                }
+                    }
+                    P += 128;
+                    V += 4 * NR;
                 }
+                nc -= t;
+                left -= t;
+                if (left > 0) break;                       // the copy is used up
+                // end of the row block: its piece
+                T* pp = part + (size_t)(warp + rb) * NR * 32 + lane;
+#pragma unroll
+                for (int j = 0; j < NR; ++j) {
+                    pp[j * 32] = acc[j] + ac2[j];
+                    acc[j] = ac2[j] = T(0);
+                }
+                if (nc + n == 0) break;                    // end of the share
+                ++rb;
+                const int r0 = R0s[rb], c0 = UP ? r0 : 0;
+                V = vin + c0 * NR;
+                left = ((UP ? W - r0 : seg_cL1(W, r0)) + 3) >> 2;
+                if (nc == 0) break;
             }
-            release(k);
+            next_slot();
         }
-        if (!waited) wait_vec(vb, par);    // a block without chunks (a slice without rows)
+        if (left > 0) {                                    // the share ends inside a row block
+            T* pp = part + (size_t)(warp + rb) * NR * 32 + lane;
 #pragma unroll
-        for (int rb = 0; rb < kRB; ++rb)
-#pragma unroll
-            for (int j = 0; j < NR; ++j) part[(warp * NR + j) * 256 + rb * 32 + lane] = acc[rb][j];
+            for (int j = 0; j < NR; ++j) pp[j * 32] = acc[j] + ac2[j];
+        }
         __syncthreads();
     };
-    // (the barrier first: owners may still be reading the previous phase's sums)
-    auto zero_part = [&]() {
-        __syncthreads();
-        for (int i = tid; i < kW * NR * 256; i += kT) part[i] = T(0);
-        __syncthreads();
-    };
-    auto part_sum = [&](int lr, int j) -> T {
-        T s = T(0);
+    const std::true_type upper{};
+    const std::false_type lower{};
+
+    // The warp's (row block, right-hand side) pairs: warp, warp + kW, ...; a lane owns a
+    // row of each.  Its right-hand side (forward) or forward result (backward) is
+    // loaded before the block product so the load is off the plane-to-plane chain.
+    int orow[NIT], oj[NIT], op[NIT], on[NIT][2];         // row, column, first piece per block type, pieces
+    bool own[NIT];
 #pragma unroll
-        for (int w = 0; w < kW; ++w) s += part[(w * NR + j) * 256 + lr];
+    for (int it = 0; it < NIT; ++it) {
+        const int k = warp + kW * it;
+        own[it] = k < nrb * nr;
+        const int rb = own[it] ? k % nrb : 0;
+        oj[it] = own[it] ? k / nrb : 0;
+        orow[it] = (own[it] ? R0s[rb] : 0) + lane;
+        const int2 u = own[it] ? pw[rb] : make_int2(0, 0), l = own[it] ? pw[kRB + rb] : make_int2(0, 0);
+        op[it] = ((u.x + rb) << 16) | (l.x + rb);
+        on[it][0] = u.y - u.x;
+        on[it][1] = l.y - l.x;
+        own[it] = own[it] && orow[it] < W;
+    }
+    // the sum of a row's pieces of an upper (t = 0) or lower (t = 1) block
+    auto psum = [&](int t, int it) -> T {
+        const T* p = part + ((t == 0 ? op[it] >> 16 : op[it] & 0xffff) * NR + oj[it]) * 32 + lane;
+        T s = p[0];
+#pragma unroll 4
+        for (int w = on[it][t]; w > 0; --w) {
+            p += NR * 32;
+            s += *p;
+        }
         return s;
     };
-
-    // Each thread owns at most one output row per plane (a slice has at most
-    // 256 rows): its right-hand side (forward) or forward result (backward) is
-    // loaded before the block product so the load is off the plane-to-plane chain.
-    int own_r = W;
-#pragma unroll
-    for (int rb = 0; rb < kRB; ++rb)
-        if ((tid >> 5) == rb) own_r = R0[rb] + (tid & 31);
-    const bool owner = tid < 32 * nrb && own_r < W;
     int ut = 0, uy = 0;        // phases of the t vector and of the y/x vector so far
     // =================================================================== forward
     for (int J = 0; J < c; ++J) {
-        const int row = J * W + own_r;
-        T pre[NR];
+        T pre[NIT];
 #pragma unroll
-        for (int j = 0; j < NR; ++j) pre[j] = (owner && row < m) ? in[b.row0 + row + j * ldi] : T(0);
-        if (J > 0) run_block(0, J, vst, &vbar[2], (uint32_t)(uy++ & 1));        // O_J y_{J-1}
-        else zero_part();
-        T* vtb = vt + (ut & 1) * NR * W;
-        if (owner) {
-#pragma unroll
-            for (int j = 0; j < NR; ++j) send(vtb, &vbar[ut & 1], j, own_r, pre[j] - part_sum(tid, j));
+        for (int it = 0; it < NIT; ++it) {
+            const int row = J * W + orow[it];
+            pre[it] = (own[it] && row < m) ? in[row0 + row + oj[it] * ldi] : T(0);
         }
+        if (J > 0) run_block(upper, vst, &vbar[2], (uint32_t)(uy++ & 1));           // O_J y_{J-1}
+        T* vtb = vt + (ut & 1) * NR * WP;
+#pragma unroll
+        for (int it = 0; it < NIT; ++it)
+            if (own[it]) send(vtb, &vbar[ut & 1], oj[it], orow[it], J > 0 ? pre[it] - psum(0, it) : pre[it]);
         arrive_local(&vbar[ut & 1]);
-        run_block(1, J, vtb, &vbar[ut & 1], (uint32_t)((ut >> 1) & 1));        // D_J t
+        run_block(lower, vtb, &vbar[ut & 1], (uint32_t)((ut >> 1) & 1));           // D_J t
         ++ut;
-        if (owner) {
 #pragma unroll
-            for (int j = 0; j < NR; ++j) {
-                const T y = part_sum(tid, j);
-                if (row < m) out[b.row0 + row + j * ldo] = y;
-                if (J + 1 < c) send(vst, &vbar[2], j, own_r, y);                 // read by O_{J+1}
+        for (int it = 0; it < NIT; ++it)
+            if (own[it]) {
+                const T y = psum(1, it);
+                if (J + 1 < c) send(vst, &vbar[2], oj[it], orow[it], y);             // read by O_{J+1}
+                const int row = J * W + orow[it];
+                if (row < m) out[row0 + row + oj[it] * ldo] = y;
             }
-        }
         if (J + 1 < c) arrive_local(&vbar[2]);
     }
     // =================================================================== backward
     for (int J = c - 1; J >= 0; --J) {
-        const int row = J * W + own_r;
-        const int64_t gi = b.row0 + row;
-        T pre[NR], bs[NR];
+        T pre[NIT], bs[NIT];
 #pragma unroll
-        for (int j = 0; j < NR; ++j) {
-            pre[j] = (owner && row < m) ? out[gi + j * ldo] : T(0);
-            bs[j] = (owner && row < m && base) ? base[gi + j * ldb] : T(0);
+        for (int it = 0; it < NIT; ++it) {
+            const int row = J * W + orow[it];
+            const bool has = own[it] && row < m;
+            pre[it] = has ? out[row0 + row + oj[it] * ldo] : T(0);
+            bs[it] = (has && base) ? base[row0 + row + oj[it] * ldb] : T(0);
         }
-        if (J < c - 1) run_block(2, J + 1, vst, &vbar[2], (uint32_t)(uy++ & 1));   // O_{J+1}^T x_{J+1}
-        else zero_part();
-        T* vtb = vt + (ut & 1) * NR * W;
-        if (owner) {
+        if (J < c - 1) run_block(lower, vst, &vbar[2], (uint32_t)(uy++ & 1));       // O_{J+1}^T x_{J+1}
+        T* vtb = vt + (ut & 1) * NR * WP;
 #pragma unroll
-            for (int j = 0; j < NR; ++j) send(vtb, &vbar[ut & 1], j, own_r, pre[j] - part_sum(tid, j));
-        }
+        for (int it = 0; it < NIT; ++it)
+            if (own[it]) send(vtb, &vbar[ut & 1], oj[it], orow[it], J < c - 1 ? pre[it] - psum(1, it) : pre[it]);
         arrive_local(&vbar[ut & 1]);
-        run_block(3, J, vtb, &vbar[ut & 1], (uint32_t)((ut >> 1) & 1));           // D_J^T t
+        run_block(upper, vtb, &vbar[ut & 1], (uint32_t)((ut >> 1) & 1));           // D_J^T t
         ++ut;
-        if (owner) {
 #pragma unroll
-            for (int j = 0; j < NR; ++j) {
-                const T x = part_sum(tid, j);
-                if (row < m) out[gi + j * ldo] = base ? bs[j] - x : x;
-                if (J > 0) send(vst, &vbar[2], j, own_r, x);                      // read by O_J^T
+        for (int it = 0; it < NIT; ++it)
+            if (own[it]) {
+                const T x = psum(0, it);
+                if (J > 0) send(vst, &vbar[2], oj[it], orow[it], x);                  // read by O_J^T
+                const int row = J * W + orow[it];
+                if (row < m) out[row0 + row + oj[it] * ldo] = base ? bs[it] - x : x;
             }
-        }
         if (J > 0) arrive_local(&vbar[2]);
     }
     cluster_barrier<G>();    // no CTA leaves while a peer may still store into it
     drain();                 // nor with a bulk copy still writing its shared memory
 }
 
-// Shared memory besides the ring (barriers, column tables, vectors, partials,
-// the ring's alignment), for planes of at most wmax rows.
+// Shared memory besides the rings (barriers, tables, vectors, pieces, the rings'
+// alignment), for planes of at most wmax rows.
 inline size_t band_fixed_bytes(int32_t wmax, int32_t nr, size_t elem, int nt) {
-    const size_t head = 2 * kMaxBuf * 8 + 4 * 8 + 2 * (kRB + 1) * 4 + 16 + 16;
-    const size_t vec = (size_t)(3 * nr * wmax + (nt / 32) * nr * 256) * elem;
-    return head + vec + 128;
+    const size_t wp = (size_t)(wmax + 3) / 4 * 4;
+    return band_head_bytes(nt) + (3 * nr * wp + (size_t)(nt / 32 + kRB) * nr * 32) * elem + 128;
 }
 
-// The ring of a CTA of nt threads: the slot count (nbuf_req, 0 for the default,
-// clamped to what fits) and the bytes per slot that fill the shared memory left
-// beside the tables and vectors; false if no ring fits.
-inline bool band_ring(int32_t wmax, int32_t nr, size_t elem, int32_t nbuf_req, int nt, int32_t* nbuf, int32_t* slot) {
+// The ring of a warp of a CTA of nt threads: the slot count (nbuf_req, 0 for the default,
+// clamped to what fits) and the quads per slot that fill the shared memory left
+// beside the tables and vectors; false if no ring fits.  Two slots: larger copies measured
+// faster than more of them (16^3 boxes, one column: FP32 103 us with two, 115 with three, 127
+// with four; FP64 362, 378, 375).
+inline bool band_ring(int32_t wmax, int32_t nr, size_t elem, int32_t nbuf_req, int nt, int32_t* nbuf, int32_t* cq) {
     const size_t fx = band_fixed_bytes(wmax, nr, elem, nt), cap = band_cap(nt);
-    if (fx + (size_t)kMinBuf * kMinSlot > cap) return false;
-    const size_t avail = cap - fx;
+    const size_t qb = 128 * elem;                                  // bytes of a quad
+    if (fx + (size_t)(nt / 32) * kMinBuf * qb > cap) return false;
+    const int32_t avail = (int32_t)((cap - fx) / (nt / 32) / qb);  // quads a warp's ring can hold
     int32_t n = nbuf_req > 0 ? nbuf_req : kDefBuf;
     n = std::max(kMinBuf, std::min<int32_t>(n, kMaxBuf));
-    while (n > kMinBuf && avail / n < (size_t)kMinSlot) --n;
+    n = std::min(n, avail);
     *nbuf = n;
-    *slot = (int32_t)((avail / n) & ~size_t(127));
+    *cq = std::min(avail / n, kMaxCq);
     return true;
 }
 
-inline size_t band_smem_bytes(int32_t wmax, int32_t nr, size_t elem, int nt, int32_t nbuf, int32_t slot) {
-    return band_fixed_bytes(wmax, nr, elem, nt) + (size_t)nbuf * slot;
+inline size_t band_smem_bytes(int32_t wmax, int32_t nr, size_t elem, int nt, int32_t nbuf, int32_t cq) {
+    return band_fixed_bytes(wmax, nr, elem, nt) + (size_t)(nt / 32) * nbuf * cq * 128 * elem;
 }
 
 namespace {
 template <typename T, int NR, int G, int NT>
 cudaError_t band_launch(const DevOperator<T>& op, int32_t p, int32_t wmax, const T* in, int64_t ldi, T* out,
-                        int64_t ldo, const T* base, int64_t ldb, cudaStream_t st) {
-    auto kern = k_band_solve2<T, NR, G, NT>;
+                        int64_t ldo, const T* base, int64_t ldb, int nr, cudaStream_t st) {
+    auto kern = k_band_wide<T, NR, G, NT>;
     // The dynamic shared-memory limit of a kernel is process-wide state on its
     // device.  It is raised once, to the device's opt-in maximum, so that
     // threads launching this kernel for operators of different widths never
@@ -570,9 +597,9 @@ cudaError_t band_launch(const DevOperator<T>& op, int32_t p, int32_t wmax, const
             raised |= 1ull << dev;
         }
     }
-    int32_t nbuf = 0, slot = 0;
-    if (!band_ring(wmax, NR, sizeof(T), op.band_nbuf, NT, &nbuf, &slot)) return cudaErrorInvalidValue;
-    const size_t smem = band_smem_bytes(wmax, NR, sizeof(T), NT, nbuf, slot);
+    int32_t nbuf = 0, cq = 0;
+    if (!band_ring(wmax, NR, sizeof(T), op.band_nbuf, NT, &nbuf, &cq)) return cudaErrorInvalidValue;
+    const size_t smem = band_smem_bytes(wmax, NR, sizeof(T), NT, nbuf, cq);
     cudaError_t e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(p * G);
@@ -586,18 +613,18 @@ cudaError_t band_launch(const DevOperator<T>& op, int32_t p, int32_t wmax, const
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = G > 1 ? 1 : 0;
-    e = cudaLaunchKernelEx(&cfg, kern, op.band, op.bfac, in, ldi, out, ldo, base, ldb, op.err, (int)nbuf, (int)slot);
+    e = cudaLaunchKernelEx(&cfg, kern, op.band, op.bfac, in, ldi, out, ldo, base, ldb, op.err, nr, (int)nbuf, (int)cq, op.bfac_len * (int64_t)sizeof(T) > kL2Keep ? 1 : 0);
     count_launches(1);
     return e;
 }
 
 template <typename T, int NR, int NT>
 cudaError_t band_launch_g(const DevOperator<T>& op, int32_t p, int32_t wmax, const T* in, int64_t ldi, T* out,
-                          int64_t ldo, const T* base, int64_t ldb, cudaStream_t st) {
+                          int64_t ldo, const T* base, int64_t ldb, int nr, cudaStream_t st) {
     switch (op.band_G) {
-        case 2: return band_launch<T, NR, 2, NT>(op, p, wmax, in, ldi, out, ldo, base, ldb, st);
-        case 4: return band_launch<T, NR, 4, NT>(op, p, wmax, in, ldi, out, ldo, base, ldb, st);
-        default: return band_launch<T, NR, 1, NT>(op, p, wmax, in, ldi, out, ldo, base, ldb, st);
+        case 2: return band_launch<T, NR, 2, NT>(op, p, wmax, in, ldi, out, ldo, base, ldb, nr, st);
+        case 4: return band_launch<T, NR, 4, NT>(op, p, wmax, in, ldi, out, ldo, base, ldb, nr, st);
+        default: return band_launch<T, NR, 1, NT>(op, p, wmax, in, ldi, out, ldo, base, ldb, nr, st);
     }
 }
 }  // namespace
@@ -605,7 +632,7 @@ cudaError_t band_launch_g(const DevOperator<T>& op, int32_t p, int32_t wmax, con
 // The 256-thread variants (instantiated in their own translation unit).
 template <typename T, int NR>
 cudaError_t band_launch_half(const DevOperator<T>& op, int32_t p, int32_t wmax, const T* in, int64_t ldi, T* out,
-                             int64_t ldo, const T* base, int64_t ldb, cudaStream_t st);
+                             int64_t ldo, const T* base, int64_t ldb, int nr, cudaStream_t st);
 
 
 }  // namespace slr

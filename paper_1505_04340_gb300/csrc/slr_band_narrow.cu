@@ -3,21 +3,20 @@
 //
 // With one slice per subdomain the factor layout is the one slr_band.cu describes:
 // row blocks 0 and 1 (rows 32 rb .. 32 rb + 31), and per block of a plane the
-// segments of 32 values (one per row) of every column that meets the triangle, row
-// blocks one after the other, columns ascending.  Warp w takes the columns
-// c = w + 4 i of every block; a lane owns rows lane and 32 + lane.
+// quads (32 rows x 4 columns) that meet the triangle, row
+// blocks one after the other, columns ascending.  Warp w takes the quads
+// w, w + 4, .. of every block (columns 4 w + 16 k + u, u < 4); a lane owns rows lane
+// and 32 + lane.
 //
 // What bounds it is the chain of 4 c - 2 small blocks (c planes), so a block is made
 // as short as the machine allows.  One CTA barrier per block:
-//   before it  each warp reads its segments of the block (they landed long ago: the
+//   before it  each warp reads its quads of the block (they landed long ago: the
 //              ring holds several whole blocks) from shared memory into registers;
 //   after it   the previous block's partial sums of all warps are visible, and the
 //              slot that every warp has just read is refilled by a fifth warp, which
 //              does nothing but issue copies.  A lane per (column, right-hand side)
 //              of its warp adds the four partial sums to the input vector's entry,
 //              which the warp keeps to itself, and the products follow from registers.
-// A column past W is multiplied like the others (its vector entry is zero), which is
-// cheaper than a test; a slot's unused end is therefore kept finite.
 // Results and right-hand sides move between a lane and global memory for the same
 // (column, right-hand side) in both passes, so the backward pass reads what its own
 // thread wrote; right-hand sides are loaded two planes ahead.
@@ -26,7 +25,7 @@
 // walking every segment in turn took 405 us.  2-D 32^2 (W = 15, FP64): 82 -> 42 us, bound
 // by the latency of 58 blocks' seven dependent FP64 operations each.
 //
-// Up to eight right-hand sides share a launch (the factor is read once).  Each sums its
+// Up to eight right-hand sides (FP64: four) share a launch (the factor is read once).  Each sums its
 // products in the same order whatever their number.  Every wait is bounded: one that
 // runs out sets the status word and the CTA's abort flag; the CTA then issues no
 // more copies and multiplies nothing, waits (bounded) for the copies it issued and
@@ -41,11 +40,12 @@ namespace {
 constexpr int kNw = 4;                      // warps per subdomain
 constexpr int kNc = 16;                     // columns of a plane a warp takes (64 / kNw)
 constexpr int kNSlots = 8;                  // ring slots at most, each a whole block
-constexpr int kNMaxR = 8;                   // right-hand sides per launch at most
+// right-hand sides per launch at most (FP64: four keep its pipe busy; eight would spill)
+template <typename T>
+constexpr int kNMaxR = sizeof(T) == 4 ? 8 : 4;
 
-// elements of a ring slot for planes of W rows: 32 values per column and row block, the
-// last row block's columns rounded up to whole groups of kNw x 4 (read, times zero)
-__host__ __device__ inline int narrow_slot(int W) { return 32 * (W <= 32 ? 32 : 96); }
+// elements of a ring slot, the largest block of a plane of W rows
+__host__ __device__ inline int narrow_slot(int W) { return 32 * (((W + 3) & ~3) + (W <= 32 ? 0 : 32)); }
 
 // NV consecutive values from shared memory (16-byte aligned)
 template <typename T, int NV>
@@ -86,11 +86,6 @@ k_band_narrow(const BandBlock* __restrict__ blocks, const T* __restrict__ fac, c
         *abort_flag = 0;
         fence_mbar_init();
     }
-    // what a block leaves of its slot is read (and multiplied by zero): it must be finite
-    const int least = min(SU, SL);
-    for (int i = tid; i < nslot * slot; i += blockDim.x)
-        if (i % slot >= least) ring[i] = T(0);
-    fence_proxy_async();
     __syncthreads();
     if (warp == kNw) {
         // ---------------------------------------------------------------- copies
@@ -142,7 +137,7 @@ k_band_narrow(const BandBlock* __restrict__ blocks, const T* __restrict__ fac, c
     T *po[NIT], *py[NIT];
 #pragma unroll
     for (int it = 0; it < NIT; ++it) {
-        const int e = it * 32 + lane, i = e % kNc, j = e / kNc, cc = warp + kNw * i;
+        const int e = it * 32 + lane, i = e % kNc, j = e / kNc, cc = 4 * warp + 16 * (i / 4) + i % 4;
         act[it] = e < kNc * NR && cc < W;
         last[it] = act[it] && cc < mlast;
         px[it] = act[it] ? j * 64 + cc : 0;
@@ -160,7 +155,7 @@ k_band_narrow(const BandBlock* __restrict__ blocks, const T* __restrict__ fac, c
     };
     int sl = 0;
     uint32_t par = 0;
-    const int coff = warp * 32 + lane;                   // first column's segment, this lane's row
+    const int coff = warp * 128 + lane * 4;              // first quad, this lane's row
     // One block: vin(it) is the entry of the input vector of the lane's pair it.
     auto step = [&](auto up, auto vin) {
         constexpr bool UP = decltype(up)::value;
@@ -176,7 +171,8 @@ k_band_narrow(const BandBlock* __restrict__ blocks, const T* __restrict__ fac, c
             }
         }
         const T* P = ring + (size_t)sl * slot + coff;
-        const T* P1 = P + 32 * (UP ? W - 32 : 32);       // row block 1: column 0 of a lower, -32 of an upper block
+        // row block 1: column 0 of a lower, -32 of an upper block
+        const T* P1 = P + 32 * (UP ? ((W + 3) & ~3) - 32 : 32);
         if (++sl == nslot) {
             sl = 0;
             par ^= 1;
@@ -184,19 +180,14 @@ k_band_narrow(const BandBlock* __restrict__ blocks, const T* __restrict__ fac, c
         T a0[N0], a1[kNc - S1];
 #pragma unroll
         for (int g = 0; g < kNc / 4; ++g) {
-            if (4 * kNw * g >= W) break;                 // columns 16 g .. 16 g + 15 of the plane
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int i = 4 * g + u;
-                if (i < N0) a0[i < N0 ? i : 0] = P[32 * kNw * i];
-            }
+            if (4 * warp + 16 * g >= W) break;           // past the plane
+            if (4 * g < N0) ld_row<T, 4>(P + 128 * kNw * g, *reinterpret_cast<T(*)[4]>(&a0[4 * g < N0 ? 4 * g : 0]));
         }
         if (two) {
 #pragma unroll
             for (int g = S1 / 4; g < kNc / 4; ++g) {
-                if (4 * kNw * g >= W) break;
-#pragma unroll
-                for (int u = 0; u < 4; ++u) a1[4 * g + u - S1] = P1[32 * kNw * (4 * g + u)];
+                if (4 * warp + 16 * g >= W) break;
+                ld_row<T, 4>(P1 + 128 * kNw * g, *reinterpret_cast<T(*)[4]>(&a1[4 * g - S1]));
             }
         }
         __syncthreads();
@@ -211,7 +202,7 @@ k_band_narrow(const BandBlock* __restrict__ blocks, const T* __restrict__ fac, c
         for (int j = 0; j < NR; ++j) acc0[j] = acc1[j] = T(0);
 #pragma unroll
         for (int g = 0; g < kNc / 4; ++g) {
-            if (4 * kNw * g >= W) break;
+            if (4 * warp + 16 * g >= W) break;
             T v[4 * NR];
             ld_row<T, 4 * NR>(vw + 4 * NR * g, v);
 #pragma unroll
@@ -353,24 +344,25 @@ cudaError_t narrow_launch(const DevOperator<T>& op, int32_t p, int32_t wmax, con
 }  // namespace
 
 // The narrow-plane band solve (planes of at most 64 rows, one slice per subdomain):
-// up to eight right-hand sides per launch.
+// up to eight (FP64: four) right-hand sides per launch.
 template <typename T>
 cudaError_t launch_band_narrow(const DevOperator<T>& op, int32_t p, int32_t wmax, const T* in, int64_t ldi, T* out,
                                int64_t ldo, const T* base, int64_t ldb, int32_t nrhs, cudaStream_t st) {
-    for (int32_t c = 0; c < nrhs; c += kNMaxR) {
+    for (int32_t c = 0; c < nrhs; c += kNMaxR<T>) {
         const T* bs = base ? base + c * ldb : nullptr;
         const T* ic = in + c * ldi;
         T* oc = out + c * ldo;
-        cudaError_t e;
-        switch (std::min(kNMaxR, nrhs - c)) {
-            case 1: e = narrow_launch<T, 1>(op, p, wmax, ic, ldi, oc, ldo, bs, ldb, st); break;
-            case 2: e = narrow_launch<T, 2>(op, p, wmax, ic, ldi, oc, ldo, bs, ldb, st); break;
-            case 3: e = narrow_launch<T, 3>(op, p, wmax, ic, ldi, oc, ldo, bs, ldb, st); break;
-            case 4: e = narrow_launch<T, 4>(op, p, wmax, ic, ldi, oc, ldo, bs, ldb, st); break;
-            case 5: e = narrow_launch<T, 5>(op, p, wmax, ic, ldi, oc, ldo, bs, ldb, st); break;
-            case 6: e = narrow_launch<T, 6>(op, p, wmax, ic, ldi, oc, ldo, bs, ldb, st); break;
-            case 7: e = narrow_launch<T, 7>(op, p, wmax, ic, ldi, oc, ldo, bs, ldb, st); break;
-            default: e = narrow_launch<T, 8>(op, p, wmax, ic, ldi, oc, ldo, bs, ldb, st); break;
+        cudaError_t e = cudaSuccess;
+        const int nr = std::min(kNMaxR<T>, nrhs - c);
+        if (nr == 1) e = narrow_launch<T, 1>(op, p, wmax, ic, ldi, oc, ldo, bs, ldb, st);
+        else if (nr == 2) e = narrow_launch<T, 2>(op, p, wmax, ic, ldi, oc, ldo, bs, ldb, st);
+        else if (nr == 3) e = narrow_launch<T, 3>(op, p, wmax, ic, ldi, oc, ldo, bs, ldb, st);
+        else if (nr == 4) e = narrow_launch<T, 4>(op, p, wmax, ic, ldi, oc, ldo, bs, ldb, st);
+        else if constexpr (sizeof(T) == 4) {
+            if (nr == 5) e = narrow_launch<T, 5>(op, p, wmax, ic, ldi, oc, ldo, bs, ldb, st);
+            else if (nr == 6) e = narrow_launch<T, 6>(op, p, wmax, ic, ldi, oc, ldo, bs, ldb, st);
+            else if (nr == 7) e = narrow_launch<T, 7>(op, p, wmax, ic, ldi, oc, ldo, bs, ldb, st);
+            else e = narrow_launch<T, 8>(op, p, wmax, ic, ldi, oc, ldo, bs, ldb, st);
         }
         if (e != cudaSuccess) return e;
     }

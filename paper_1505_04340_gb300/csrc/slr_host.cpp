@@ -329,12 +329,12 @@ void host_band_layout(HostSetup& hs, int32_t G) {
                 std::memcpy(b.rbmap, it->second.rbmap, sizeof(b.rbmap));
             }
         }
-        int so = 0, sd = 0;   // segments of the widest slice
+        int so = 0, sd = 0;   // columns (whole quads) of the widest slice
         for (int g = 0; g < G; ++g) {
             int a = 0, d = 0;
             for (int rb = 0; rb < b.nrb[g]; ++rb) {
-                a += b.w - band_cU0(b, g, rb);
-                d += band_cL1(b, g, rb);
+                a += band_c4(b.w - band_cU0(b, g, rb));
+                d += band_c4(band_cL1(b, g, rb));
             }
             so = std::max(so, a);
             sd = std::max(sd, d);
@@ -418,25 +418,30 @@ slr_status host_band_factor(HostSetup& hs, int32_t G) {
                 double* Lf = Uf + b.SU;                                 // D_J      (lower)
                 double* Lb = Lf + b.SL;                                 // O_J^T    (lower)
                 double* Ub = Lb + b.SL;                                 // D_J^T    (upper)
-                int64_t su = 0, sl = 0;   // next upper / lower segment
+                int64_t su = 0, sl = 0;   // the row block's first upper / lower column
                 for (int rb = 0; rb < b.nrb[g]; ++rb) {
                     const int R0 = band_R0(b, g, rb);
-                    for (int cc = band_cU0(b, g, rb); cc < W; ++cc, ++su)      // upper: rows r <= cc
+                    const int cu0 = band_cU0(b, g, rb), cl1 = band_cL1(b, g, rb);
+                    for (int cc = cu0; cc < W; ++cc)                           // upper: rows r <= cc
                         for (int e = 0; e < 32; ++e) {
                             const int r = R0 + e, l = J * W + r;
+                            const int64_t at = su * 32 + band_elem(cc - cu0, e);
                             if (r >= W || r > cc) continue;
                             // forward blocks carry the pivot signs: O_J S_{J-1} and S_J D_J^{-1}
-                            Uf[su * 32 + e] = (J > 0 && l < m) ? Lat(l, (J - 1) * W + cc) * sg[(size_t)(J - 1) * W + cc]
+                            Uf[at] = (J > 0 && l < m) ? Lat(l, (J - 1) * W + cc) * sg[(size_t)(J - 1) * W + cc]
                                                                : 0.0;                            // O_J[r][cc]
-                            Ub[su * 32 + e] = X[(size_t)cc * W + r];                             // D_J^{-1}[cc][r]
+                            Ub[at] = X[(size_t)cc * W + r];                             // D_J^{-1}[cc][r]
                         }
-                    for (int cc = 0; cc < band_cL1(b, g, rb); ++cc, ++sl)      // lower: rows r >= cc
+                    for (int cc = 0; cc < cl1; ++cc)                           // lower: rows r >= cc
                         for (int e = 0; e < 32; ++e) {
                             const int r = R0 + e, lc = J * W + cc;
+                            const int64_t at = sl * 32 + band_elem(cc, e);
                             if (r >= W || r < cc) continue;
-                            Lf[sl * 32 + e] = X[(size_t)r * W + cc] * sg[(size_t)J * W + r];     // D_J^{-1}[r][cc]
-                            Lb[sl * 32 + e] = (J > 0 && lc < m) ? Lat(lc, (J - 1) * W + r) : 0.0;   // O_J[cc][r]
+                            Lf[at] = X[(size_t)r * W + cc] * sg[(size_t)J * W + r];     // D_J^{-1}[r][cc]
+                            Lb[at] = (J > 0 && lc < m) ? Lat(lc, (J - 1) * W + r) : 0.0;   // O_J[cc][r]
                         }
+                    su += band_c4(W - cu0);
+                    sl += band_c4(cl1);
                 }
             }
         }

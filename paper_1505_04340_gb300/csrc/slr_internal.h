@@ -22,8 +22,9 @@ namespace slr {
 // cluster (slices) each own whole blocks, assigned so that the slices' shares
 // of upper-block and lower-block work are even (band_assign_blocks); slice g's
 // local row block rb is block rbmap[g][rb].  A slice of a block is tiled: for
-// every (local row block, column) pair that meets the triangle, one segment of
-// 32 values (zero outside the triangle and past W), row blocks one after the
+// every (local row block, four columns) that meet the triangle, one "quad" of 32 x 4
+// values, row e's four columns together (one 16-byte FP32 load per lane; zero
+// outside the triangle and past W), row blocks one after the
 // other, columns ascending.  Per plane and slice: [O_J | D_J | O_J^T | D_J^T] =
 // [SU | SL | SL | SU] elements; a plane occupies G * 2 (SU + SL).  The last plane
 // is padded with identity rows.  (Shared with slr_band.cu.)
@@ -33,8 +34,8 @@ struct BandBlock {
     int32_t c = 0;        // planes, c * W >= m
     int32_t row0 = 0;     // first row of B_i inside u (DD interior order)
     int64_t foff = 0;     // offset of plane 0 in the factor array (elements)
-    int32_t SU = 0;       // elements of one upper slice block (32 per segment, widest slice)
-    int32_t SL = 0;       // elements of one lower slice block (32 per segment, widest slice)
+    int32_t SU = 0;       // elements of one upper slice block (128 per quad, widest slice)
+    int32_t SL = 0;       // elements of one lower slice block (128 per quad, widest slice)
     int32_t id = 0;       // the subdomain i (blocks may be launched in another order)
     uint8_t nrb[4] = {0, 0, 0, 0};   // row blocks of each slice (at most 8: 256 rows)
     uint8_t rbmap[4][8] = {};        // block of slice g's local row block rb
@@ -57,6 +58,10 @@ inline int band_cU0(const BandBlock& b, int g, int rb) { return std::min(b.w, ba
 inline int band_cL1(const BandBlock& b, int g, int rb) {
     return std::min(b.w, std::min(band_R0(b, g, rb) + 31, b.w - 1) + 1);
 }
+// Columns rounded up to whole quads, and the element of (column k of a row block's
+// columns, row e of the row block) from the row block's first quad on.
+inline int band_c4(int cols) { return (cols + 3) & ~3; }
+inline int64_t band_elem(int k, int e) { return (int64_t)(k >> 2) * 128 + e * 4 + (k & 3); }
 // True if G slices can hold a plane of W rows (at most 8 blocks of 32 rows each).
 inline bool band_split_ok(int W, int G) { return (W + 31) / 32 <= 8 * G; }
 // Deal the 32-row blocks of a plane of b.w rows to G slices (fills nrb, rbmap).
