@@ -19,12 +19,14 @@
 // One CTA of 256 threads per subdomain, three roles:
 //   thread 0 (warp 0)  streams the sub-tiles through a ring of shared slots with
 //                      1-D bulk copies (cp.async.bulk) on "full" mbarriers;
-//   thread 32 (warp 1) issues the MMAs of a block once its vector operand is in
-//                      shared memory, returns each slot by tcgen05.commit on its
-//                      "empty" mbarrier and signals the accumulator on "acc";
+//   warp 1             issues the MMAs of a block once its vector operand is in
+//                      shared memory (one elected lane), returns each slot by
+//                      tcgen05.commit on its "empty" mbarrier and signals the
+//                      accumulator on "acc";
 //   warps 4-7          read the accumulator (thread e owns rows e and 128 + e),
-//                      form t, Y or X, write the next operand into shared memory
-//                      and the results to global memory, and arrive on "opnd".
+//                      form t, Y or X, write the next operand into shared memory,
+//                      arrive on "opnd", and then write the results to global memory
+//                      (the next block has the other accumulators).
 // Every wait is bounded: one that runs out sets the status word (1) and the CTA's
 // abort flag; every role then stops, thread 0 waits (bounded) for the copies it
 // issued, thread 32 for the MMAs it issued, and the tensor memory is freed.
@@ -184,6 +186,8 @@ __device__ __forceinline__ void bt_put_rows(unsigned char* vdst, int rbase, int 
     }
 }
 
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 template <int AB, int NP>
 __global__ void __launch_bounds__(kBtThreads, NP <= 32 ? 2 : 1)
 k_band_tc(const BandTcBlock* __restrict__ blocks, const unsigned char* __restrict__ fac, const float* in,
@@ -212,14 +216,15 @@ k_band_tc(const BandTcBlock* __restrict__ blocks, const unsigned char* __restric
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tbase + 1);
     const int tid = threadIdx.x, warp = tid >> 5;
     const int nM = (W + 127) / 128;
-    // tensor memory: the accumulators (M-tile mt at column mt CS), then as many columns
+    // tensor memory: the accumulators (M-tile mt at column mt CS) of even and of odd
+    // blocks, then as many columns as one of them
     // holding the epilogue's global operand of a block (F_J, Y_J or the base), written
     // by the epilogue threads while the block's MMAs run.  The epilogue moves 32
     // columns at a time, so an M-tile's columns are at least 32 wide (CS): with N = 16
     // and two M-tiles, a stride of 16 would put the second tile's staged operand past
     // the allocation, into the columns of the SM's other CTA.
     constexpr uint32_t CS = NP < 32 ? 32 : NP;
-    const uint32_t acols = nM * CS <= 32 ? 32 : nM * CS <= 64 ? 64 : 128, ncol = 2 * acols;
+    const uint32_t acols = nM * CS <= 32 ? 32 : nM * CS <= 64 ? 64 : 128, ncol = 4 * acols;   // (a power of two)
     if (warp == 0) {
         tc::tmem_alloc(tbase, ncol);
         tc::tmem_relinquish();
@@ -252,6 +257,8 @@ k_band_tc(const BandTcBlock* __restrict__ blocks, const unsigned char* __restric
 
     if (tid == 0) {
         // ---------------------------------------------------------------- producer
+        uint64_t pol;                                   // the factor leaves L2 first: it is read once per pass
+        asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
         int f = 0, s = 0;                               // copies issued, slot of the next one
         uint32_t par = 1;                               // parity of the slot's last release
         for (int q = 0; q < nblk && !*abort_flag; ++q) {
@@ -270,9 +277,9 @@ k_band_tc(const BandTcBlock* __restrict__ blocks, const unsigned char* __restric
                              "r"(bytes)
                              : "memory");
                 asm volatile(
-                    "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                    "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;" ::"r"(
                         tc::smem_addr(ring + (size_t)s * stiles * kSub)),
-                    "l"(src + (int64_t)t0 * kSub), "r"(bytes), "r"(tc::smem_addr(&full[s]))
+                    "l"(src + (int64_t)t0 * kSub), "r"(bytes), "r"(tc::smem_addr(&full[s])), "l"(pol)
                     : "memory");
                 if (++s == nslot) {
                     s = 0;
@@ -286,12 +293,16 @@ k_band_tc(const BandTcBlock* __restrict__ blocks, const unsigned char* __restric
             const int last = s + ((f - 1 - s) / nslot) * nslot;
             tc::mbar_wait(&full[s], (uint32_t)((last / nslot) & 1), kBtSpin);
         }
-    } else if (tid == 32) {
+    } else if (warp == 1) {
         // ---------------------------------------------------------------- MMA issuer
-        // One thread issues every MMA, so its instructions are the block's critical path:
-        // the slot, its parity and both descriptors are carried along instead of being
-        // formed anew for each sub-tile (with two divisions and a modulo per sub-tile an
-        // MMA took 540 cycles to issue, 24,000 of a block's 28,000; the MMA itself takes about 20).
+        // The instructions around an MMA are a block's critical path: with a slot, a parity and
+        // two descriptors formed anew for each sub-tile by one thread an MMA took 540 cycles to
+        // issue, 24,000 of a block's 28,000; the MMA itself keeps its pipe busy for about 20.  So
+        // the warp stays converged and one elected lane issues, a slot's sub-tiles of an
+        // M-tile in one unrolled run from descriptors that are carried along: 7,000 cycles of
+        // a block's 11,500.  (Storing only the sub-tiles' rows inside the triangle and
+        // masking the rest saved 36% of the bytes and no time; an issuer per M-tile neither.)
+        const bool elected = tc::elect_one();
         const uint32_t idesc = tc::instr_desc(AB, 128, NP);
         const uint64_t ring_desc = tc::smem_desc(tc::smem_addr(ring), 128, 256);
         const uint64_t vec_desc = tc::smem_desc(tc::smem_addr(vbuf), 128, sbo_v);
@@ -306,28 +317,31 @@ k_band_tc(const BandTcBlock* __restrict__ blocks, const unsigned char* __restric
             tc::fence_after_sync();
             // the operand: t (D blocks) or Y / X (O blocks), written by the last epilogue
             int left = tiles_of(bk.type), in_slot = 0;  // sub-tiles of the block, of the slot
-            uint64_t ad = 0;
             bool ok = true;
             for (int mt = 0; mt < nM && ok; ++mt) {
                 const int k0 = bt_k0(upper, mt, KS), k1 = bt_k1(upper, mt, W, KS);
-                const uint32_t d = tmem + (uint32_t)(mt * CS);
-                uint64_t bd = vec_desc + kStepDesc * k0;
-                for (int ks = k0; ks < k1; ++ks) {
-                    if (in_slot == 0) {
-                        if (!tc::mbar_wait(&full[s], par, kBtSpin)) {
-                            fail();
-                            ok = false;
-                            break;
-                        }
-                        ad = ring_desc + kSubDesc * (uint32_t)(s * stiles);
+                const uint32_t d = tmem + (uint32_t)(q & 1) * acols + (uint32_t)(mt * CS);
+                for (int ks = k0; ks < k1;) {
+                    if (in_slot == 0 && !tc::mbar_wait(&full[s], par, kBtSpin)) {
+                        fail();
+                        ok = false;
+                        break;
                     }
-                    tc::mma<AB>(d, ad, bd, idesc, ks > k0);
-                    ad += kSubDesc;
-                    bd += kStepDesc;
-                    ++in_slot;
-                    --left;
+                    // the sub-tiles of this M-tile in the slot
+                    const int n = min(stiles - in_slot, k1 - ks);
+                    const uint64_t ad = ring_desc + kSubDesc * (uint32_t)(s * stiles + in_slot);
+                    const uint64_t bd = vec_desc + kStepDesc * (uint32_t)ks;
+                    if (elected) {
+                        tc::mma<AB>(d, ad, bd, idesc, ks > k0);
+#pragma unroll
+                        for (int i = 1; i < 8; ++i)
+                            if (i < n) tc::mma<AB>(d, ad + kSubDesc * i, bd + kStepDesc * i, idesc, true);
+                    }
+                    ks += n;
+                    in_slot += n;
+                    left -= n;
                     if (in_slot == stiles || left == 0) {       // the slot's last sub-tile
-                        tc::commit(&empty[s]);
+                        if (elected) tc::commit(&empty[s]);
                         in_slot = 0;
                         if (++s == nslot) {
                             s = 0;
@@ -337,16 +351,14 @@ k_band_tc(const BandTcBlock* __restrict__ blocks, const unsigned char* __restric
                 }
             }
             if (!ok) break;
-            tc::commit(acc_bar);
+            if (elected) tc::commit(acc_bar);
         }
-        tc::commit(fin_bar);                            // every MMA issued has completed
+        if (elected) tc::commit(fin_bar);                            // every MMA issued has completed
         tc::mbar_wait(fin_bar, 0, kBtSpin);
     } else if (warp >= 4) {
         // ---------------------------------------------------------------- epilogue
         const int e = tid - 128, quarter = warp - 4;
         const uint32_t lane_addr = (uint32_t)(32 * quarter) << 16;
-        unsigned char* v0 = vbuf;                       // Y / X
-        unsigned char* v1 = vbuf;                       // t (the same buffer, in turn)
         // byte of (column j, row r) of an operand (K index r)
         auto opos = [&](int j, int r) -> uint32_t {
             return (uint32_t)((j >> 3) * sbo_v + (r / (16 / E)) * 128 + (j & 7) * 16 + (r % (16 / E)) * E);
@@ -364,7 +376,7 @@ k_band_tc(const BandTcBlock* __restrict__ blocks, const unsigned char* __restric
             if (r >= W) continue;
             const bool ok = valid(0, r);
             for (int j = 0; j < nrhs; ++j)
-                *reinterpret_cast<Te*>(v1 + opos(j, r)) = Tp::pack(ok ? in[row_of(0, r) + j * ldi] : 0.0f);
+                *reinterpret_cast<Te*>(vbuf + opos(j, r)) = Tp::pack(ok ? in[row_of(0, r) + j * ldi] : 0.0f);
         }
         arrive();
         auto put_rows = [&](unsigned char* vdst, int rbase, int c0, const float (&v)[32]) {
@@ -377,6 +389,19 @@ k_band_tc(const BandTcBlock* __restrict__ blocks, const unsigned char* __restric
             // previous block's epilogue, by these threads, has read the columns)
             const bool need_pre = bk.type == 0 || bk.type == 2 || (bk.type == 3 && base);
             if (need_pre) {
+                // the plane that the next block of this type will want, into L2
+                const int Jn = bk.type == 0 ? J + 1 : J - 1;
+                if (Jn >= 0 && Jn < c) {
+                    const float* src = bk.type == 0 ? in : bk.type == 2 ? out : base;
+                    const int64_t lds = bk.type == 0 ? ldi : bk.type == 2 ? ldo : ldb;
+                    for (int mt = 0; mt < nM; ++mt) {
+                        const int r0 = 128 * mt + 32 * quarter;
+                        for (int j = tid & 31; j < nrhs; j += 32) {
+                            if (valid(Jn, r0)) prefetch_l2(src + row_of(Jn, r0) + j * lds);
+                            if (valid(Jn, r0 + 31)) prefetch_l2(src + row_of(Jn, r0 + 31) + j * lds);
+                        }
+                    }
+                }
                 const float* srcb = bk.type == 0 ? in : bk.type == 2 ? out : base;
                 const int64_t lds = bk.type == 0 ? ldi : bk.type == 2 ? ldo : ldb;
                 for (int mt = 0; mt < nM; ++mt) {
@@ -389,7 +414,7 @@ k_band_tc(const BandTcBlock* __restrict__ blocks, const unsigned char* __restric
 #pragma unroll
                         for (int jj = 0; jj < 32; ++jj)
                             pv[jj] = (ok && c0 + jj < nrhs) ? srcb[row + (c0 + jj) * lds] : 0.0f;
-                        tc::tmem_st32(tmem + lane_addr + acols + (uint32_t)(mt * CS + c0), pv);
+                        tc::tmem_st32(tmem + lane_addr + 2 * acols + (uint32_t)(mt * CS + c0), pv);
                     }
                 }
             }
@@ -401,58 +426,56 @@ k_band_tc(const BandTcBlock* __restrict__ blocks, const unsigned char* __restric
             }
             if (__any_sync(0xffffffffu, *abort_flag != 0)) break;
             tc::fence_after_sync();
-            for (int mt = 0; mt < nM; ++mt) {
-                const int r = 128 * mt + e;
-                const bool in_w = r < W, ok_r = valid(J, r);
-                const int64_t row = row_of(J, r);
-                const int rbase = 128 * mt + 32 * quarter;      // first row of the warp
+            // first the next block's operand, so that its MMAs can start; the results go to
+            // global memory after that (the next block has the other accumulators)
+            const uint32_t acc = tmem + lane_addr + (uint32_t)(q & 1) * acols;
+            const uint32_t pre = tmem + lane_addr + 2 * acols;
+            if (q + 1 < nblk) {
+                for (int mt = 0; mt < nM; ++mt) {
+                    const int rbase = 128 * mt + 32 * quarter;      // first row of the warp
 #pragma unroll
-                for (int c0 = 0; c0 < NP; c0 += 32) {
-                    float v[32];
-                    tc::tmem_ld32(tmem + lane_addr + (uint32_t)(mt * CS + c0), v);
-                    const uint32_t pre_col = tmem + lane_addr + acols + (uint32_t)(mt * CS + c0);
-                    // v := pre - v (the operand's columns past nrhs were stored as zeros)
-                    auto pre_minus = [&]() {
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            float p[16];
-                            tc::tmem_ld16(pre_col + 16 * h, p);
-#pragma unroll
-                            for (int i = 0; i < 16; ++i) v[16 * h + i] = p[i] - v[16 * h + i];
-                        }
-                    };
-                    if (bk.type == 0 || bk.type == 2) {          // t = F_J - O_J Y_{J-1}  /  Y_J - O^T X
-                        pre_minus();
-                        put_rows(v1, rbase, c0, v);
-                    } else if (bk.type == 1) {                   // Y_J = D_J t
-                        if (in_w && ok_r) {
-#pragma unroll
-                            for (int jj = 0; jj < 32; ++jj)
-                                if (c0 + jj < nrhs) out[row + (c0 + jj) * ldo] = v[jj];
-                        }
-                        put_rows(v0, rbase, c0, v);             // also the backward's first t (J = c - 1)
-                    } else {                                     // X_J = D_J^T t (out: base - X_J with a base)
-                        if (base) {
+                    for (int c0 = 0; c0 < NP; c0 += 32) {
+                        float v[32];
+                        tc::tmem_ld32(acc + (uint32_t)(mt * CS + c0), v);
+                        if (bk.type == 0 || bk.type == 2) {          // t = F_J - O_J Y_{J-1}  /  Y_J - O^T X
+                            // (the operand's columns past nrhs were stored as zeros)
 #pragma unroll
                             for (int h = 0; h < 2; ++h) {
                                 float p[16];
-                                tc::tmem_ld16(pre_col + 16 * h, p);    // warp-collective: every lane
-                                if (in_w && ok_r) {
+                                tc::tmem_ld16(pre + (uint32_t)(mt * CS + c0) + 16 * h, p);
 #pragma unroll
-                                    for (int i = 0; i < 16; ++i)
-                                        if (c0 + 16 * h + i < nrhs) out[row + (c0 + 16 * h + i) * ldo] = p[i] - v[16 * h + i];
-                                }
+                                for (int i = 0; i < 16; ++i) v[16 * h + i] = p[i] - v[16 * h + i];
                             }
-                        } else if (in_w && ok_r) {
-#pragma unroll
-                            for (int jj = 0; jj < 32; ++jj)
-                                if (c0 + jj < nrhs) out[row + (c0 + jj) * ldo] = v[jj];
                         }
-                        put_rows(v0, rbase, c0, v);
+                        put_rows(vbuf, rbase, c0, v);                // Y_J, X_J (also the backward's first t) or t
+                    }
+                }
+                arrive();
+            }
+            if (bk.type == 1 || bk.type == 3) {                      // Y_J = D_J t / X_J = D_J^T t (base - X_J)
+                for (int mt = 0; mt < nM; ++mt) {
+                    const int r = 128 * mt + e;
+                    const bool ok_r = valid(J, r);
+                    const int64_t row = row_of(J, r);
+#pragma unroll
+                    for (int c0 = 0; c0 < NP; c0 += 32) {
+                        float v[32];
+                        tc::tmem_ld32(acc + (uint32_t)(mt * CS + c0), v);
+                        const bool sub = bk.type == 3 && base;
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            float p[16];
+                            if (sub) tc::tmem_ld16(pre + (uint32_t)(mt * CS + c0) + 16 * h, p);   // warp-collective
+                            if (ok_r) {
+#pragma unroll
+                                for (int i = 0; i < 16; ++i)
+                                    if (c0 + 16 * h + i < nrhs)
+                                        out[row + (c0 + 16 * h + i) * ldo] = sub ? p[i] - v[16 * h + i] : v[16 * h + i];
+                            }
+                        }
                     }
                 }
             }
-            if (q + 1 < nblk) arrive();
         }
     }
     tc::fence_before_sync();
@@ -470,11 +493,11 @@ cudaError_t bt_launch(const DevOperator<float>& op, int32_t p, const float* in, 
     const int WK = bt_nk(op.band_tc_wmax, KS) * KS;
     const size_t vbytes = (size_t)NP * WK * E;
     const size_t fixed = vbytes + 8 * (2 * 8 + 3) + 16;
-    // ring: as many 8-sub-tile slots (32 KB) as fit, 2 .. 8, in the opt-in maximum or,
+    // ring: as many 4-sub-tile slots (16 KB) as fit, 2 .. 8, in the opt-in maximum or,
     // with more subdomains than SMs, in half an SM (113 KB: two CTAs per SM, one wave).
-    // Fewer, larger copies measured faster: on 3-D 96^3 with 32 columns two 32 KB slots
-    // took 1014 us per B-solve, five of 16 KB 1039 us, ten of 8 KB 1114 us.
-    const int stiles = 8;
+    // 3-D 96^3, 32 columns, one B-solve with its two conversions: 522 us with five slots of
+    // 16 KB, 526 with two of 32 KB, 529 with six of 12 KB.
+    const int stiles = 4;
     const size_t cap = (NP <= 32 && p > op.cf.nsm) ? 113 * 1024 : 227 * 1024;
     int nslot = fixed < cap ? (int)((cap - fixed) / ((size_t)stiles * kSub)) : 0;
     nslot = nslot > 8 ? 8 : nslot;
