@@ -395,54 +395,73 @@ __device__ __forceinline__ void ld4(const T* p, T (&v)[4]) {
     }
 }
 
-// Forward task on a block of RP right-hand sides j0 .. j0 + nb - 1 in one pass (RP 16
-// or 32; columns past nb are zeros): t_J from the level's gather, stored right-hand
+// Forward task on a block of RP right-hand sides j0 .. j0 + nb - 1 in one pass (columns
+// past nb are zeros): t_J from the level's gather, stored right-hand
 // sides contiguous with row stride RP + 4 (16-byte loads by the lanes of different
-// columns then meet distinct banks).  Panel rows: a warp per row, lanes over the
-// columns with RP sums each, then one reduce-scatter; diagonal rows: lane = row, the
+// columns then meet distinct banks).  Panel rows: a warp takes R of them, lanes over the
+// columns with R x RP sums each, then a reduce-scatter per row.  One row at a time read eight
+// 16-byte words of t_J for 32 multiply-adds, four times what the shared memory delivers
+// beside them; four rows of 16 right-hand sides read four for 64, as much as the
+// FP32 units take.  Diagonal rows: lane = row, the
 // warps split the columns and their partial sums are added in order.  Every (row,
 // right-hand side) gets the multiply-adds and additions of cfwd_task_rb, bit for bit.
 // red2: NW x RP x 32.
-template <typename T, int NW, int RP>
+template <typename T, int NW, int RP, int R>
 __device__ void cfwd_task_blk(const CView<T>& cf, const int4 tk, bool pan, T* ts, T* red2, T* xf, int j0, int nb) {
     constexpr int RS = RP + 4;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int32_t J = tk.x, a0 = cf.c0[J], nJ = cf.c0[J + 1] - a0;
     const int ncl = pan ? nJ : tk.y + tk.z;        // columns the task reads
+    const T* P = cf.panel + cf.pan_off[J];
+    const int64_t w0 = cf.r_off[J];
     for (int idx = threadIdx.x; idx < ncl * RP; idx += NW * 32) {
         const int i = idx / RP, b = idx - i * RP;     // right-hand sides fastest: contiguous in the gather
         ts[i * RS + b] = b < nb ? cf.tws[(int64_t)(a0 + i) * cf.wr + j0 + b] : T(0);
     }
     __syncthreads();
     if (pan) {
-        const T* P = cf.panel + cf.pan_off[J];
-        for (int pr = warp; pr < tk.z; pr += NW) {
-            const int64_t p = tk.y + pr;
-            const T* Pp = P + p * nJ;
-            T acc[RP];
+        for (int pr = warp * R; pr < tk.z; pr += NW * R) {
+            const T* Pp[R];
 #pragma unroll
-            for (int b = 0; b < RP; ++b) acc[b] = T(0);
-            auto madd = [&](T a, int c) {
+            for (int r = 0; r < R; ++r) Pp[r] = P + (int64_t)(tk.y + min(pr + r, tk.z - 1)) * nJ;
+            T acc[R][RP];
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+#pragma unroll
+                for (int b = 0; b < RP; ++b) acc[r][b] = T(0);
+            auto madd = [&](const T (&a)[R], int c) {
 #pragma unroll
                 for (int q = 0; q < RP; q += 4) {
                     T t4[4];
                     ld4(ts + c * RS + q, t4);
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) acc[q + e] += a * t4[e];
+                    for (int r = 0; r < R; ++r)
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) acc[r][q + e] += a[r] * t4[e];
                 }
             };
+            // the next columns' entries are in flight during a step's products
+            T a[R], an[R];
             int c = lane;
-            for (; c + 7 * 32 < nJ; c += 8 * 32) {
-                T pv[8];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) pv[u] = Pp[c + 32 * u];
+            for (int r = 0; r < R; ++r) an[r] = c < nJ ? Pp[r][c] : T(0);
+            for (; c < nJ; c += 32) {
 #pragma unroll
-                for (int u = 0; u < 8; ++u) madd(pv[u], c + 32 * u);
+                for (int r = 0; r < R; ++r) a[r] = an[r];
+                if (c + 32 < nJ) {
+#pragma unroll
+                    for (int r = 0; r < R; ++r) an[r] = Pp[r][c + 32];
+                }
+                madd(a, c);
             }
-            for (; c < nJ; c += 32) madd(Pp[c], c);
-            const T v = reduce_scatter<T, RP>(acc, lane);
-            const int k = rs_index<RP>(lane);
-            if (rs_writer<RP>(lane) && k < nb) cf.wbuf[(cf.r_off[J] + p) * cf.wr + j0 + k] = v;
+            __syncwarp();
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const T v = reduce_scatter<T, RP>(acc[r], lane);
+                const int k = rs_index<RP>(lane);
+                if (rs_writer<RP>(lane) && k < nb && pr + r < tk.z)
+                    cf.wbuf[(w0 + tk.y + pr + r) * cf.wr + j0 + k] = v;
+            }
         }
     } else {
         const T* D = cf.dinv + cf.dinv_off[J];
@@ -592,26 +611,36 @@ __device__ void cbwd_task_rb(const CView<T>& cf, const int4 tk, T* us, T (*red)[
 
 // Backward task on a block of RP right-hand sides j0 .. j0 + nb - 1 in one pass: the
 // diagonal part as in cbwd_task_rb (a warp per column, lanes over the rows) with RP
-// sums per lane and one reduce-scatter; the panel part with lanes over the columns
-// and the warps splitting the panel rows, each warp staging the gathered rows of
-// x_{R_J} (32 rows x RP, one right-hand side per lane, row stride RP + 4) in its own
-// part of xs and reading them back by 16-byte broadcasts; its
+// sums per lane and one reduce-scatter, y_J's rows from the task's first column on
+// staged in ys (row stride RP + 4, ystage; from global memory otherwise); the panel
+// part with lanes over the columns and the warps splitting the panel rows, each warp
+// gathering 32 rows of x_{R_J} at a time into its own part of xs (row stride RP + 4)
+// and reading them back by 16-byte broadcasts.  A batch costs two latencies: its row
+// numbers are loaded during the batch before it, all its rows of x at once, and the
+// panel's entries eight rows ahead of their products.  The
 // partial sums then go to xs (the same buffer) and are added over the warps in
 // order.  Every column gets cbwd_task_rb's multiply-adds and additions, bit for bit.
 // us: RP x 32; xs: NW x 32 x (RP + 4).
 template <typename T, int NW, int RP>
-__device__ void cbwd_task_blk(const CView<T>& cf, const int4 tk, T* us, T* xs, const T* yf, T* xf, T* y_dd,
-                              int64_t ldy, int j0, int nb) {
-    constexpr int RS = RP + 4;
+__device__ void cbwd_task_blk(const CView<T>& cf, const int4 tk, T* us, T* xs, T* ys, bool ystage, const T* yf, T* xf,
+                              T* y_dd, int64_t ldy, int j0, int nb) {
+    constexpr int RS = RP + 4, NG = 32 / RP > 0 ? 32 / RP : 1;   // rows a warp gathers at once
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int32_t J = tk.x, a0 = cf.c0[J], nJ = cf.c0[J + 1] - a0, jl = tk.y + lane;
     const int64_t nr = cf.r_off[J + 1] - cf.r_off[J];
     const int32_t* R = cf.rows + cf.r_off[J];
-    const T* Pn = cf.panel + cf.pan_off[J] + jl;
+    const T* Pn = cf.panel + cf.pan_off[J] + (lane < tk.z ? jl : tk.y);
     const T* D = cf.dinv + cf.dinv_off[J];
     const int64_t chunk = (nr + NW - 1) / NW, pb = warp * chunk, pe = min(nr, pb + chunk);
     const T* y = yf + a0 + (int64_t)j0 * cf.s;
     const T* x = xf + j0;                    // x(pos, b) at x[pos xr + b]
+    int32_t rnext = pb + lane < pe ? R[pb + lane] : 0;
+    if (ystage) {
+        for (int b = warp; b < RP; b += NW)
+            for (int i = tk.y + lane; i < nJ; i += 32)
+                ys[(i - tk.y) * RS + b] = b < nb ? y[(int64_t)b * cf.s + i] : T(0);
+        __syncthreads();
+    }
     // right-hand side b of the block (zero past nb)
     auto yv = [&](int b, int64_t i) { return b < nb ? y[(int64_t)b * cf.s + i] : T(0); };
     for (int cc = warp; cc < tk.z; cc += NW) {
@@ -621,20 +650,34 @@ __device__ void cbwd_task_blk(const CView<T>& cf, const int4 tk, T* us, T* xs, c
 #pragma unroll
         for (int b = 0; b < RP; ++b) acc[b] = T(0);
         int i = c + lane;
-        for (; i + 7 * 32 < nJ; i += 8 * 32) {
-            T d[8];
+        if (ystage) {
+            const T* yi = ys + (i - tk.y) * RS;
+            auto madd = [&](T d) {
 #pragma unroll
-            for (int u = 0; u < 8; ++u) d[u] = Dc[i + 32 * u];
+                for (int q = 0; q < RP; q += 4) {
+                    T t4[4];
+                    ld4(yi + q, t4);
 #pragma unroll
-            for (int u = 0; u < 8; ++u)
+                    for (int e = 0; e < 4; ++e) acc[q + e] += d * t4[e];
+                }
+                yi += 32 * RS;
+            };
+            for (; i + 3 * 32 < nJ; i += 4 * 32) {
+                T d[4];
 #pragma unroll
-                for (int b = 0; b < RP; ++b) acc[b] += d[u] * yv(b, i + 32 * u);
+                for (int u = 0; u < 4; ++u) d[u] = Dc[i + 32 * u];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) madd(d[u]);
+            }
+            for (; i < nJ; i += 32) madd(Dc[i]);
+        } else {
+            for (; i < nJ; i += 32) {
+                const T d = Dc[i];
+#pragma unroll
+                for (int b = 0; b < RP; ++b) acc[b] += d * yv(b, i);
+            }
         }
-        for (; i < nJ; i += 32) {
-            const T d = Dc[i];
-#pragma unroll
-            for (int b = 0; b < RP; ++b) acc[b] += d * yv(b, i);
-        }
+        __syncwarp();
         const T v = reduce_scatter<T, RP>(acc, lane);
         if (rs_writer<RP>(lane)) us[rs_index<RP>(lane) * 32 + cc] = v;
     }
@@ -642,30 +685,47 @@ __device__ void cbwd_task_blk(const CView<T>& cf, const int4 tk, T* us, T* xs, c
 #pragma unroll
     for (int b = 0; b < RP; ++b) acc[b] = T(0);
     T* xw = xs + (size_t)warp * 32 * RS;               // this warp's rows
+    const int gb = lane % RP, gr = lane / RP;          // the right-hand side and row a lane gathers
     for (int64_t q0 = pb; q0 < pe; q0 += 32) {
         const int nq = (int)min((int64_t)32, pe - q0);
-        // x_{R_J} rows q0 .. q0 + nq - 1: lane b loads right-hand side b of each
-        if (lane < RP) {
-            T v[8];
-            for (int pp0 = 0; pp0 < nq; pp0 += 8) {
+        const T* Pq = Pn + q0 * nJ;
+        T pv[8];
 #pragma unroll
-                for (int u = 0; u < 8; ++u)
-                    v[u] = (pp0 + u < nq && lane < nb) ? x[(int64_t)R[q0 + pp0 + u] * cf.xr + lane] : T(0);
+        for (int u = 0; u < 8; ++u) pv[u] = u < nq ? Pq[(int64_t)u * nJ] : T(0);
+        // x_{R_J} rows q0 .. q0 + nq - 1
+        const int32_t r = rnext;
+        rnext = q0 + 32 + lane < pe ? R[q0 + 32 + lane] : 0;
 #pragma unroll
-                for (int u = 0; u < 8; ++u)
-                    if (pp0 + u < nq) xw[(pp0 + u) * RS + lane] = v[u];
+        for (int h = 0; h < 2; ++h) {
+            T v[16 / NG];
+#pragma unroll
+            for (int u = 0; u < 16 / NG; ++u) {
+                const int row = 16 * h + u * NG + gr;
+                const int32_t pos = __shfl_sync(0xffffffffu, r, row & 31);
+                v[u] = (row < nq && gb < nb && gr < NG) ? x[(int64_t)pos * cf.xr + gb] : T(0);
             }
+#pragma unroll
+            for (int u = 0; u < 16 / NG; ++u)
+                if (gr < NG) xw[(16 * h + u * NG + gr) * RS + gb] = v[u];
         }
         __syncwarp();
-        if (lane < tk.z) {
-            for (int pp = 0; pp < nq; ++pp) {
-                const T pv = Pn[(q0 + pp) * nJ];
+        for (int p0 = 0; p0 < nq; p0 += 8) {
+            T pc[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) pc[u] = pv[u];
+            if (p0 + 8 < nq) {
+#pragma unroll
+                for (int u = 0; u < 8; ++u) pv[u] = p0 + 8 + u < nq ? Pq[(int64_t)(p0 + 8 + u) * nJ] : T(0);
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                if (p0 + u >= nq) break;
 #pragma unroll
                 for (int q = 0; q < RP; q += 4) {
                     T t4[4];
-                    ld4(xw + pp * RS + q, t4);
+                    ld4(xw + (p0 + u) * RS + q, t4);
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) acc[q + e] += pv * t4[e];
+                    for (int e = 0; e < 4; ++e) acc[q + e] += pc[u] * t4[e];
                 }
             }
         }
@@ -1222,18 +1282,20 @@ k_cfwd_level(const CView<T> cf, int32_t t0, int32_t p0, int32_t np, const T* g, 
                          nrhs, red2);
 }
 
-// forward level, blocks of right-hand sides in passes of RP (cfwd_task_blk); dynamic
-// shared memory: t_J (tstride x (RP + 4)), then NW x RP x 32 partial sums
-template <typename T, int NW, int RP>
+// forward level, blocks of right-hand sides: CTA (q, y) runs task q on the y-th group of RP
+// right-hand sides (cfwd_task_blk; more CTAs for the levels of few tasks, and less
+// shared memory each); dynamic shared memory: t_J (tstride x (RP + 4)), then NW x RP x 32
+// partial sums
+template <typename T, int NW, int RP, int R>
 __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 1)
 k_cfwd_level_blk(const CView<T> cf, int32_t t0, int32_t p0, int32_t np, T* xf, int32_t nrhs, int32_t tstride) {
     extern __shared__ __align__(16) unsigned char csm[];
-    const int q = blockIdx.x;
+    const int q = blockIdx.x, j0 = blockIdx.y * RP;
     const bool pan = q < np;
     T* ts = reinterpret_cast<T*>(csm);
     T* red2 = ts + (size_t)tstride * (RP + 4);
     const int4 tk = pan ? cf.ptasks[p0 + q] : cf.tasks[t0 + q - np];
-    for (int j0 = 0; j0 < nrhs; j0 += RP) cfwd_task_blk<T, NW, RP>(cf, tk, pan, ts, red2, xf, j0, min(RP, nrhs - j0));
+    cfwd_task_blk<T, NW, RP, R>(cf, tk, pan, ts, red2, xf, j0, min(RP, nrhs - j0));
 }
 
 // gf[ciperm[i] wr + j] = g[i + j ldg]: the forward's input in factor order, a row per position.
@@ -1288,17 +1350,19 @@ k_cbwd_level(const CView<T> cf, int32_t t0, const T* yf, T* xf, T* y_dd, int64_t
                                                       nrhs, red2);
 }
 
-// backward level, blocks of right-hand sides in passes of RP (cbwd_task_blk); dynamic
-// shared memory: us (RP x 32), then xs (NW x 32 x (RP + 4))
+// backward level, blocks of right-hand sides: CTA (q, y) runs task q on the y-th group of RP
+// right-hand sides (cbwd_task_blk); dynamic shared memory: us (RP x 32), xs (NW x 32 x
+// (RP + 4)), then (ystage) y_J (the level's widest supernode x (RP + 4))
 template <typename T, int NW, int RP>
 __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 1)
-k_cbwd_level_blk(const CView<T> cf, int32_t t0, const T* yf, T* xf, T* y_dd, int64_t ldy, int32_t nrhs) {
+k_cbwd_level_blk(const CView<T> cf, int32_t t0, const T* yf, T* xf, T* y_dd, int64_t ldy, int32_t nrhs, int ystage) {
     extern __shared__ __align__(16) unsigned char csm[];
     T* us = reinterpret_cast<T*>(csm);
     T* xs = us + RP * 32;
+    T* ys = xs + (size_t)NW * 32 * (RP + 4);
     const int4 tk = cf.tasks[t0 + blockIdx.x];
-    for (int j0 = 0; j0 < nrhs; j0 += RP)
-        cbwd_task_blk<T, NW, RP>(cf, tk, us, xs, yf, xf, y_dd, ldy, j0, min(RP, nrhs - j0));
+    const int j0 = blockIdx.y * RP;
+    cbwd_task_blk<T, NW, RP>(cf, tk, us, xs, ys, ystage != 0, yf, xf, y_dd, ldy, j0, min(RP, nrhs - j0));
 }
 
 // right-hand sides per pass of the fused small levels' per-level kernels
@@ -2143,35 +2207,26 @@ cudaError_t launch_c_forward(const DevCFactor<T>& cf, const T* g_dd, int64_t ldg
             counted();
         }
         const bool wide = nt + np <= cf.nsm;
-        // blocks of 8 or more with the level's gather: one pass per 32 (16 in the wide
-        // variant, 8 when the level's widest supernode leaves no room for 16) right-hand
-        // sides when t_J of that many fits; every variant forms the same sums in the same order
+        // blocks of 8 or more with the level's gather: a CTA per task and 16 (8 when there are
+        // no more, or when the level's widest supernode leaves no room for 16) right-hand
+        // sides; every variant forms the same sums in the same order.  3-D 96^3, 32 columns: the
+        // eight narrow levels took 485 us in passes of 32 with a row per warp, 362 us now
         if (nrhs >= 8 && vl.tws) {
             const int32_t ts_n = cf.lev_maxn[l] > 0 ? cf.lev_maxn[l] : cf.max_n;
-            auto smem_for = [&](int rp, int nw) { return ((size_t)ts_n * (rp + 4) + (size_t)nw * rp * 32) * sizeof(T); };
-            auto fits = [&](size_t sm, const void* kb) {
-                return sm <= kLevSmem && (sm <= 48 * 1024 || raise_smem_once(kb));
+            auto blk = [&](auto kern, int rp, int nw) -> bool {
+                const size_t sm = ((size_t)ts_n * (rp + 4) + (size_t)nw * rp * 32) * sizeof(T);
+                if (sm > kLevSmem || (sm > 48 * 1024 && !raise_smem_once((const void*)kern))) return false;
+                kern<<<dim3(nt + np, (nrhs + rp - 1) / rp), nw * 32, sm, st>>>(vl, t0, p0, np, xf, nrhs, ts_n);
+                counted();
+                return true;
             };
+            constexpr int R = sizeof(T) == 4 ? 4 : 2;      // panel rows per warp (registers)
             if (!wide) {
-                const size_t sm = smem_for(32, 8);
-                if (fits(sm, (const void*)k_cfwd_level_blk<T, 8, 32>)) {
-                    k_cfwd_level_blk<T, 8, 32><<<nt + np, 256, sm, st>>>(vl, t0, p0, np, xf, nrhs, ts_n);
-                    counted();
-                    continue;
-                }
+                if (nrhs > 8 && blk(k_cfwd_level_blk<T, 8, 16, R>, 16, 8)) continue;
+                if (blk(k_cfwd_level_blk<T, 8, 8, 4>, 8, 8)) continue;
             } else {
-                size_t sm = smem_for(16, 32);
-                if (fits(sm, (const void*)k_cfwd_level_blk<T, 32, 16>)) {
-                    k_cfwd_level_blk<T, 32, 16><<<nt + np, 1024, sm, st>>>(vl, t0, p0, np, xf, nrhs, ts_n);
-                    counted();
-                    continue;
-                }
-                sm = smem_for(8, 32);
-                if (fits(sm, (const void*)k_cfwd_level_blk<T, 32, 8>)) {
-                    k_cfwd_level_blk<T, 32, 8><<<nt + np, 1024, sm, st>>>(vl, t0, p0, np, xf, nrhs, ts_n);
-                    counted();
-                    continue;
-                }
+                if (nrhs > 8 && blk(k_cfwd_level_blk<T, 32, 16, 1>, 16, 32)) continue;
+                if (blk(k_cfwd_level_blk<T, 32, 8, 1>, 8, 32)) continue;
             }
         }
         // blocks of eight or four right-hand sides share each matrix load when t_J of that many fits
@@ -2231,22 +2286,27 @@ cudaError_t launch_c_backward(const DevCFactor<T>& cf, const T* yf, T* xf, T* y_
         }
         const int t0 = cf.lev_task_ptr[l], nt = cf.lev_task_ptr[l + 1] - t0;
         if (nt == 0) continue;
-        if (nrhs >= 8) {                               // blocks of 8 or more: one pass per 32 (16 wide)
+        if (nrhs >= 8) {                               // blocks of 8 or more: a CTA per task and 16 (or 8) of them
+            // (3-D 96^3, 32 columns: the nine levels 380 us, 645 with y_J read from global memory for
+            // each column, a panel entry's load waiting for the one before, and passes in turn)
             const bool wide = nt <= cf.nsm;
+            const int32_t mn = cf.lev_maxn[l] > 0 ? cf.lev_maxn[l] : cf.max_n;
+            auto blk = [&](auto kern, int rp, int nw) -> bool {
+                const size_t base = ((size_t)rp * 32 + (size_t)nw * 32 * (rp + 4)) * sizeof(T);
+                const size_t full = base + (size_t)mn * (rp + 4) * sizeof(T);
+                const bool ystage = full <= kLevSmem;
+                const size_t sm = ystage ? full : base;
+                if (sm > kLevSmem || (sm > 48 * 1024 && !raise_smem_once((const void*)kern))) return false;
+                kern<<<dim3(nt, (nrhs + rp - 1) / rp), nw * 32, sm, st>>>(v, t0, yf, xf, y_dd, ldy, nrhs, ystage ? 1 : 0);
+                counted();
+                return true;
+            };
             if (!wide) {
-                const size_t sm = ((size_t)32 * 32 + (size_t)8 * 32 * 36) * sizeof(T);
-                if (sm <= 48 * 1024 || raise_smem_once((const void*)k_cbwd_level_blk<T, 8, 32>)) {
-                    k_cbwd_level_blk<T, 8, 32><<<nt, 256, sm, st>>>(v, t0, yf, xf, y_dd, ldy, nrhs);
-                    counted();
-                    continue;
-                }
+                if (nrhs > 8 && blk(k_cbwd_level_blk<T, 8, 16>, 16, 8)) continue;
+                if (blk(k_cbwd_level_blk<T, 8, 8>, 8, 8)) continue;
             } else {
-                const size_t sm = ((size_t)16 * 32 + (size_t)32 * 32 * 20) * sizeof(T);
-                if (sm <= 48 * 1024 || raise_smem_once((const void*)k_cbwd_level_blk<T, 32, 16>)) {
-                    k_cbwd_level_blk<T, 32, 16><<<nt, 1024, sm, st>>>(v, t0, yf, xf, y_dd, ldy, nrhs);
-                    counted();
-                    continue;
-                }
+                if (nrhs > 8 && blk(k_cbwd_level_blk<T, 32, 16>, 16, 32)) continue;
+                if (blk(k_cbwd_level_blk<T, 32, 8>, 8, 32)) continue;
             }
         }
         // blocks of four or more: the panel part's partial sums, NW x 8 x 32
