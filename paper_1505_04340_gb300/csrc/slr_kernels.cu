@@ -20,6 +20,8 @@
 
 namespace slr {
 
+bool raise_smem_once(const void* kern);
+
 std::atomic<int64_t> g_kernel_launches{0};
 thread_local int64_t t_kernel_launches = 0;
 
@@ -1365,41 +1367,60 @@ k_cbwd_level_blk(const CView<T> cf, int32_t t0, const T* yf, T* xf, T* y_dd, int
     cbwd_task_blk<T, NW, RP>(cf, tk, us, xs, ys, ystage != 0, yf, xf, y_dd, ldy, j0, min(RP, nrhs - j0));
 }
 
-// right-hand sides per pass of the fused small levels' per-level kernels
-constexpr int kSmallRBf = 8, kSmallRBb = 4;
-
-// dynamic shared memory: t_J (tsz elements: kSmallRBf right-hand sides, or tile_rp
-// contiguous ones for the tiled path of blocks of 8 or more), then the stage buffer
-// of cap elements
-template <typename T>
+// Fused small levels, one launch per level.  RB right-hand sides per pass of the narrow paths:
+// as many as the call has (1, 2, 4, forward also 8), since each costs its multiply-adds whether
+// it is there or not, and FP64's are slow (one FP64 column on 3-D 64^3 with RB = 8 forward and 4
+// backward spent 190 us of a 1228 us apply on absent columns).  Blocks of 8 or more take the
+// tiled paths.
+// dynamic shared memory: t_J (tsz elements: RB right-hand sides, or tile_rp
+// contiguous ones for the tiled path), then the stage buffer of cap elements
+template <typename T, int RB>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 2)
-k_cfwd_small(const CView<T> cf, int32_t s0, const T* g, int64_t ldg, T* xf, int32_t nrhs, int32_t cap, int32_t tsz) {
-    extern __shared__ __align__(16) unsigned char csm[];
-    T* ts = reinterpret_cast<T*>(csm);
-    cfwd_small_cta<T, kThreads, 1, kSmallRBf>(cf, cf.lev_sn[s0 + blockIdx.x], ts, g, ldg, xf, nrhs, ts + tsz, cap,
-                                              tsz == kSmallN * tile_rp<T>());
-}
-
-// dynamic shared memory (vsz elements): kSmallRBb vectors of kSmallN + kSmallR and
-// kSmallRBb x kThreads partial sums, or for blocks of 8 or more the tiled path's
-// buffer, then the stage buffer of cap elements
-template <typename T>
-__host__ __device__ constexpr int small_bwd_vsz(bool tiled) {
-    return tiled ? (tile_vs<T>() > kSmallRBb * (kSmallN + kSmallR + kThreads) ? tile_vs<T>()
-                                                                              : kSmallRBb * (kSmallN + kSmallR + kThreads))
-                 : kSmallRBb * (kSmallN + kSmallR + kThreads);
-}
-template <typename T>
-__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 2)
-k_cbwd_small(const CView<T> cf, int32_t s0, const T* yf, T* xf, T* y_dd, int64_t ldy, int32_t nrhs, int32_t cap,
+k_cfwd_small(const CView<T> cf, int32_t s0, const T* g, int64_t ldg, T* xf, int32_t nrhs, int32_t cap, int32_t tsz,
              bool tiled) {
     extern __shared__ __align__(16) unsigned char csm[];
-    T* vs = reinterpret_cast<T*>(csm);
-    T* red = vs + kSmallRBb * (kSmallN + kSmallR);
-    cbwd_small_cta<T, kThreads, 1, kSmallRBb>(cf, cf.lev_sn[s0 + blockIdx.x], vs, red, yf, xf, y_dd, ldy, nrhs,
-                                              vs + small_bwd_vsz<T>(tiled), cap, tiled);
+    T* ts = reinterpret_cast<T*>(csm);
+    cfwd_small_cta<T, kThreads, 1, RB>(cf, cf.lev_sn[s0 + blockIdx.x], ts, g, ldg, xf, nrhs, ts + tsz, cap, tiled);
 }
 
+// dynamic shared memory (vsz elements): RB vectors of kSmallN + kSmallR and
+// RB x kThreads partial sums, or for blocks of 8 or more the tiled path's
+// buffer if that is more, then the stage buffer of cap elements
+template <typename T, int RB>
+__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 2)
+k_cbwd_small(const CView<T> cf, int32_t s0, const T* yf, T* xf, T* y_dd, int64_t ldy, int32_t nrhs, int32_t cap,
+             int32_t vsz, bool tiled) {
+    extern __shared__ __align__(16) unsigned char csm[];
+    T* vs = reinterpret_cast<T*>(csm);
+    T* red = vs + RB * (kSmallN + kSmallR);
+    cbwd_small_cta<T, kThreads, 1, RB>(cf, cf.lev_sn[s0 + blockIdx.x], vs, red, yf, xf, y_dd, ldy, nrhs, vs + vsz, cap,
+                                       tiled);
+}
+
+template <typename T, int RB>
+cudaError_t cfwd_small_launch(const CView<T>& v, int s0, int ns, int32_t cap, const T* g, int64_t ldg, T* xf,
+                              int32_t nrhs, cudaStream_t st) {
+    const bool tiled = nrhs >= 8;
+    const int32_t tsz = tiled ? kSmallN * tile_rp<T>() : RB * kSmallN;
+    const size_t sm = ((size_t)tsz + cap) * sizeof(T);
+    auto kern = k_cfwd_small<T, RB>;
+    if (sm > 48 * 1024 && !raise_smem_once((const void*)kern)) return cudaErrorInvalidValue;
+    kern<<<ns, kThreads, sm, st>>>(v, s0, g, ldg, xf, nrhs, cap, tsz, tiled);
+    count_launches(1);
+    return cudaGetLastError();
+}
+template <typename T, int RB>
+cudaError_t cbwd_small_launch(const CView<T>& v, int s0, int ns, int32_t cap, const T* yf, T* xf, T* y_dd, int64_t ldy,
+                              int32_t nrhs, cudaStream_t st) {
+    const bool tiled = nrhs >= 8;
+    const int32_t plain = RB * (kSmallN + kSmallR + kThreads), vsz = tiled ? std::max(tile_vs<T>(), plain) : plain;
+    const size_t sm = ((size_t)vsz + cap) * sizeof(T);
+    auto kern = k_cbwd_small<T, RB>;
+    if (sm > 48 * 1024 && !raise_smem_once((const void*)kern)) return cudaErrorInvalidValue;
+    kern<<<ns, kThreads, sm, st>>>(v, s0, yf, xf, y_dd, ldy, nrhs, cap, vsz, tiled);
+    count_launches(1);
+    return cudaGetLastError();
+}
 
 // ---- top zone: x_T = L_TT^{-1} t_T and y_T = L_TT^{-T} x_T with the explicit inverse
 // (local index la of the zone's positions; tpos maps it to the factor order)
@@ -2187,11 +2208,12 @@ cudaError_t launch_c_forward(const DevCFactor<T>& cf, const T* g_dd, int64_t ldg
             const int s0 = cf.lev_sn_ptr[l], ns = cf.lev_sn_ptr[l + 1] - s0;
             if (ns == 0) continue;
             const int32_t cap = cf.lev_stage[l];
-            const int32_t tsz = nrhs >= 8 ? kSmallN * tile_rp<T>() : kSmallRBf * kSmallN;
-            const size_t sm = ((size_t)tsz + cap) * sizeof(T);
-            if (sm > 48 * 1024 && !raise_smem_once((const void*)k_cfwd_small<T>)) return cudaErrorInvalidValue;
-            k_cfwd_small<T><<<ns, kThreads, sm, st>>>(v, s0, g_dd, ldg, xf, nrhs, cap, tsz);
-            counted();
+            const cudaError_t e =
+                nrhs == 1   ? cfwd_small_launch<T, 1>(v, s0, ns, cap, g_dd, ldg, xf, nrhs, st)
+                : nrhs == 2 ? cfwd_small_launch<T, 2>(v, s0, ns, cap, g_dd, ldg, xf, nrhs, st)
+                : nrhs <= 4 ? cfwd_small_launch<T, 4>(v, s0, ns, cap, g_dd, ldg, xf, nrhs, st)
+                            : cfwd_small_launch<T, 8>(v, s0, ns, cap, g_dd, ldg, xf, nrhs, st);
+            if (e != cudaSuccess) return e;
             continue;
         }
         const int t0 = cf.lev_task_ptr[l], nt = cf.lev_task_ptr[l + 1] - t0;
@@ -2277,11 +2299,11 @@ cudaError_t launch_c_backward(const DevCFactor<T>& cf, const T* yf, T* xf, T* y_
             const int s0 = cf.lev_sn_ptr[l], ns = cf.lev_sn_ptr[l + 1] - s0;
             if (ns == 0) continue;
             const int32_t cap = cf.lev_stage[l];
-            const bool tiled = nrhs >= 8;
-            const size_t sm = ((size_t)small_bwd_vsz<T>(tiled) + cap) * sizeof(T);
-            if (sm > 48 * 1024 && !raise_smem_once((const void*)k_cbwd_small<T>)) return cudaErrorInvalidValue;
-            k_cbwd_small<T><<<ns, kThreads, sm, st>>>(v, s0, yf, xf, y_dd, ldy, nrhs, cap, tiled);
-            counted();
+            const cudaError_t e =
+                nrhs == 1   ? cbwd_small_launch<T, 1>(v, s0, ns, cap, yf, xf, y_dd, ldy, nrhs, st)
+                : nrhs == 2 ? cbwd_small_launch<T, 2>(v, s0, ns, cap, yf, xf, y_dd, ldy, nrhs, st)
+                            : cbwd_small_launch<T, 4>(v, s0, ns, cap, yf, xf, y_dd, ldy, nrhs, st);
+            if (e != cudaSuccess) return e;
             continue;
         }
         const int t0 = cf.lev_task_ptr[l], nt = cf.lev_task_ptr[l + 1] - t0;
