@@ -1426,15 +1426,16 @@ cudaError_t cbwd_small_launch(const CView<T>& v, int s0, int ns, int32_t cap, co
 // (local index la of the zone's positions; tpos maps it to the factor order)
 constexpr int kTopT = 256;   // threads of the zone kernels (8 warps)
 
-// t_T = g_T - (panel products of the supernodes below the zone), one thread per (la, j)
+// t_T = g_T - (panel products of the supernodes below the zone), one thread per (la, j), the
+// right-hand sides fastest (a gathered row of w is one line)
 template <typename T>
 __global__ void __launch_bounds__(kThreads)
 k_ctop_gather(const CView<T> cf, const T* g, int64_t ldg, int32_t nrhs) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (int64_t)cf.nT * nrhs) return;
-    const int32_t la = (int32_t)(i % cf.nT), j = (int32_t)(i / cf.nT);
-    cf.tT[i] = g_at(cf, cf.tpos[la], g, ldg, j) -
-               gather_sum(cf.wbuf + j, cf.wr, cf.tseg_row, cf.tseg_ptr[la], cf.tseg_ptr[la + 1]);
+    const int32_t la = (int32_t)(i / nrhs), j = (int32_t)(i - (int64_t)la * nrhs);
+    cf.tT[la + (int64_t)j * cf.nT] = g_at(cf, cf.tpos[la], g, ldg, j) -
+                                     gather_sum(cf.wbuf + j, cf.wr, cf.tseg_row, cf.tseg_ptr[la], cf.tseg_ptr[la + 1]);
 }
 
 // Adds the chunks' partial sums of a block once all its tasks have stored theirs:
@@ -1461,13 +1462,18 @@ __device__ __forceinline__ void last_task_sum(int32_t* cnt, int nch, const T* pa
     if (threadIdx.x == 0) *cnt = 0;
 }
 
-// forward task (row block rb, columns [cb, ce), chunk k): partial sums of rows
-// r0 .. r0 + count - 1 of L_TT^{-1} t_T over the chunk; a warp takes rows
-// w, w + 8, w + 16, w + 24 (four in flight), lanes over the columns
+// Right-hand sides per pass of the zone kernels at most: the inverse's entries are read once for them.
 template <typename T>
+constexpr int kTopR = sizeof(T) == 4 ? 8 : 4;
+
+// forward task (row block rb, columns [cb, ce), chunk k): partial sums of rows
+// r0 .. r0 + count - 1 of L_TT^{-1} t_T over the chunk for RB right-hand sides at a time; a warp
+// takes rows w, w + 8, w + 16, w + 24 (four in flight), lanes over the columns; the 4 x RB sums
+// over the lanes by one reduce-scatter (warp_sum's tree)
+template <typename T, int RB>
 __global__ void __launch_bounds__(kTopT)
 k_ctop_fwd(const CView<T> cf, T* xf, int32_t nrhs) {
-    __shared__ T ts[kTopCW];
+    __shared__ T ts[RB][kTopCW];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int4 tk = cf.tf_tasks[blockIdx.x];
     const int4 rb = cf.tf_rb[tk.x];
@@ -1479,11 +1485,17 @@ k_ctop_fwd(const CView<T> cf, T* xf, int32_t nrhs) {
         la[u] = r < rb.y ? rb.x + r : -1;
         off[u] = r < rb.y ? cf.tsk_off[la[u]] - cf.tsk_lo[la[u]] : 0;
     }
-    for (int j = 0; j < nrhs; ++j) {
-        const T* t = cf.tT + (int64_t)j * cf.nT;
-        for (int c = tk.y + threadIdx.x; c < tk.z; c += kTopT) ts[c - tk.y] = t[c];
+    for (int j0 = 0; j0 < nrhs; j0 += RB) {
+        const int nb = min(RB, nrhs - j0);
+#pragma unroll
+        for (int b = 0; b < RB; ++b) {
+            const T* t = cf.tT + (int64_t)(j0 + min(b, nb - 1)) * cf.nT;
+            for (int c = tk.y + threadIdx.x; c < tk.z; c += kTopT) ts[b][c - tk.y] = t[c];
+        }
         __syncthreads();
-        T acc[4] = {T(0), T(0), T(0), T(0)};
+        T acc[4 * RB];
+#pragma unroll
+        for (int q = 0; q < 4 * RB; ++q) acc[q] = T(0);
         int c = tk.y + lane;
         // sixteen loads in flight per lane (four rows x four columns); entries right
         // of a row's diagonal, and rows past the block, load nothing
@@ -1494,24 +1506,28 @@ k_ctop_fwd(const CView<T> cf, T* xf, int32_t nrhs) {
 #pragma unroll
                 for (int q = 0; q < 4; ++q) a[u][q] = c + 32 * q <= la[u] ? cf.tsk[off[u] + c + 32 * q] : T(0);
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const T tv = ts[c + 32 * q - tk.y];
+            for (int q = 0; q < 4; ++q)
 #pragma unroll
-                for (int u = 0; u < 4; ++u) acc[u] += a[u][q] * tv;
-            }
+                for (int b = 0; b < RB; ++b) {
+                    const T tv = ts[b][c + 32 * q - tk.y];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) acc[u * RB + b] += a[u][q] * tv;
+                }
         }
         for (; c < tk.z; c += 32) {
-            const T tv = ts[c - tk.y];
 #pragma unroll
             for (int u = 0; u < 4; ++u)
-                if (c <= la[u]) acc[u] += cf.tsk[off[u] + c] * tv;
-        }
+                if (c <= la[u]) {
+                    const T a = cf.tsk[off[u] + c];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const T v = warp_sum(acc[u]);
-            if (lane == 0 && la[u] >= 0)
-                cf.tf_part[(int64_t)j * cf.tf_parts + rb.w + tk.w * 32 + warp + 8 * u] = v;
+                    for (int b = 0; b < RB; ++b) acc[u * RB + b] += a * ts[b][c - tk.y];
+                }
         }
+        __syncwarp();
+        const T v = reduce_scatter<T, 4 * RB>(acc, lane);
+        const int k = rs_index<4 * RB>(lane), u = k / RB, b = k % RB;
+        if (rs_writer<4 * RB>(lane) && b < nb && warp + 8 * u < rb.y)
+            cf.tf_part[(int64_t)(j0 + b) * cf.tf_parts + rb.w + tk.w * 32 + warp + 8 * u] = v;
         __syncthreads();
     }
     last_task_sum(cf.tf_cnt + tk.x, rb.z, cf.tf_part + rb.w, cf.tf_parts, rb.y, nrhs,
@@ -1519,15 +1535,15 @@ k_ctop_fwd(const CView<T> cf, T* xf, int32_t nrhs) {
 }
 
 // backward task (column block cb of J, path rows [r0, r1), chunk k): partial sums of
-// columns c0 .. c0 + count - 1 of X_J^T x over the chunk (lanes over the columns,
-// the warps split the rows, 16 (FP32) or 8 (FP64) loads in flight); the chunk's x
-// values are staged in shared memory
-template <typename T>
+// columns c0 .. c0 + count - 1 of X_J^T x over the chunk for RB right-hand sides at a time (lanes
+// over the columns, the warps split the rows, 16 (FP32) or 8 (FP64) loads in flight); the
+// chunk's x values are staged in shared memory, right-hand sides contiguous
+template <typename T, int RB>
 __global__ void __launch_bounds__(kTopT)
 k_ctop_bwd(const CView<T> cf, const T* yf, T* xf, T* y_dd, int64_t ldy, int32_t nrhs) {
     constexpr int NW = kTopT / 32, DEPTH = sizeof(T) == 4 ? 16 : 8;
-    __shared__ T xs[kTopRCH];
-    __shared__ T red[NW][33];
+    __shared__ __align__(16) T xs[kTopRCH * RB];
+    __shared__ T red[NW][RB][33];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int4 tk = cf.tb_tasks[blockIdx.x];
     const int4 cb = cf.tb_cb[tk.x];
@@ -1536,29 +1552,52 @@ k_ctop_bwd(const CView<T> cf, const T* yf, T* xf, T* y_dd, int64_t ldy, int32_t 
     const int32_t* pp = cf.tp_pos + cf.tp_off[J];
     const int nrw = tk.z - tk.y, per = (nrw + NW - 1) / NW;
     const int rb = tk.y + warp * per, re = min(tk.z, rb + per);
-    for (int j = 0; j < nrhs; ++j) {
-        for (int r = tk.y + threadIdx.x; r < tk.z; r += kTopT) xs[r - tk.y] = yf[pp[r] + (int64_t)j * cf.s];
+    for (int j0 = 0; j0 < nrhs; j0 += RB) {
+        const int nb = min(RB, nrhs - j0);
+        for (int r = tk.y + threadIdx.x; r < tk.z; r += kTopT) {
+            const T* y = yf + pp[r] + (int64_t)j0 * cf.s;
+#pragma unroll
+            for (int b = 0; b < RB; ++b) xs[(r - tk.y) * RB + b] = b < nb ? y[(int64_t)b * cf.s] : T(0);
+        }
         __syncthreads();
-        T acc = T(0);
+        T acc[RB];
+#pragma unroll
+        for (int b = 0; b < RB; ++b) acc[b] = T(0);
         if (lane < cb.z) {
+            auto madd = [&](T a, int r) {
+                const T* x = xs + (r - tk.y) * RB;
+#pragma unroll
+                for (int q = 0; q < RB; q += RB < 4 ? 1 : 4) {
+                    if constexpr (RB < 4) {
+                        acc[q] += a * x[q];
+                    } else {
+                        T t4[4];
+                        ld4(x + q, t4);
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) acc[q + e] += a * t4[e];
+                    }
+                }
+            };
             int r = rb;
             for (; r + DEPTH - 1 < re; r += DEPTH) {
                 T a[DEPTH];
 #pragma unroll
                 for (int u = 0; u < DEPTH; ++u) a[u] = X[(int64_t)(r + u) * nJ];
 #pragma unroll
-                for (int u = 0; u < DEPTH; ++u) acc += a[u] * xs[r + u - tk.y];
+                for (int u = 0; u < DEPTH; ++u) madd(a[u], r + u);
             }
-            for (; r < re; ++r) acc += X[(int64_t)r * nJ] * xs[r - tk.y];
+            for (; r < re; ++r) madd(X[(int64_t)r * nJ], r);
         }
-        red[warp][lane] = acc;
-        __syncthreads();
-        if (warp == 0 && lane < cb.z) {
-            T v = T(0);
 #pragma unroll
-            for (int w = 0; w < NW; ++w) v += red[w][lane];
-            cf.tb_part[(int64_t)j * cf.tb_parts + pofs + tk.w * 32 + lane] = v;
-        }
+        for (int b = 0; b < RB; ++b) red[warp][b][lane] = acc[b];
+        __syncthreads();
+        for (int b = warp; b < nb; b += NW)
+            if (lane < cb.z) {
+                T v = T(0);
+#pragma unroll
+                for (int w = 0; w < NW; ++w) v += red[w][b][lane];
+                cf.tb_part[(int64_t)(j0 + b) * cf.tb_parts + pofs + tk.w * 32 + lane] = v;
+            }
         __syncthreads();
     }
     const int32_t a0 = cf.c0[J] + cb.y;
@@ -2284,7 +2323,10 @@ cudaError_t launch_c_forward(const DevCFactor<T>& cf, const T* g_dd, int64_t ldg
     }
     if (cf.nT > 0) {
         k_ctop_gather<T><<<blocks_for((int64_t)cf.nT * nrhs), kThreads, 0, st>>>(v, g_dd, ldg, nrhs);
-        k_ctop_fwd<T><<<cf.n_tf_tasks, kTopT, 0, st>>>(v, xf, nrhs);
+        if (nrhs == 1) k_ctop_fwd<T, 1><<<cf.n_tf_tasks, kTopT, 0, st>>>(v, xf, nrhs);
+        else if (nrhs == 2) k_ctop_fwd<T, 2><<<cf.n_tf_tasks, kTopT, 0, st>>>(v, xf, nrhs);
+        else if (nrhs <= 4) k_ctop_fwd<T, 4><<<cf.n_tf_tasks, kTopT, 0, st>>>(v, xf, nrhs);
+        else k_ctop_fwd<T, kTopR<T>><<<cf.n_tf_tasks, kTopT, 0, st>>>(v, xf, nrhs);
         counted(2);
     }
     return cudaGetLastError();
@@ -2297,7 +2339,10 @@ cudaError_t launch_c_backward(const DevCFactor<T>& cf, const T* yf, T* xf, T* y_
     CView<T> v = make_view(cf, cf.nsteps_bwd);
     v.xr = nrhs;     // the solution x (scratch): a call's right-hand sides contiguous per row
     if (cf.nT > 0) {
-        k_ctop_bwd<T><<<cf.n_tb_tasks, kTopT, 0, st>>>(v, yf, xf, y_dd, ldy, nrhs);
+        if (nrhs == 1) k_ctop_bwd<T, 1><<<cf.n_tb_tasks, kTopT, 0, st>>>(v, yf, xf, y_dd, ldy, nrhs);
+        else if (nrhs == 2) k_ctop_bwd<T, 2><<<cf.n_tb_tasks, kTopT, 0, st>>>(v, yf, xf, y_dd, ldy, nrhs);
+        else if (nrhs <= 4) k_ctop_bwd<T, 4><<<cf.n_tb_tasks, kTopT, 0, st>>>(v, yf, xf, y_dd, ldy, nrhs);
+        else k_ctop_bwd<T, kTopR<T>><<<cf.n_tb_tasks, kTopT, 0, st>>>(v, yf, xf, y_dd, ldy, nrhs);
         counted();
     }
     if (cf.nsteps_bwd == 0) return cudaGetLastError();
