@@ -205,7 +205,7 @@ slr_status upload_operator(slr_handle h, DevOperator<T>& op, bool with_band) {
     // 36 KB (the rest of the 48 KB default holds the kernels' static arrays); the
     // forward stages the panel with an odd row stride (n_J | 1), so sizes count it
     {
-        const int64_t capmax = 36 * 1024 / (int64_t)sizeof(T);
+        const int64_t capmax = 56 * 1024 / (int64_t)sizeof(T), perscap = 36 * 1024 / (int64_t)sizeof(T);
         d.lev_stage.assign(c.nlev, 0);
         d.stage_cap = 0;
         for (int32_t l = 0; l < c.nlev; ++l) {
@@ -217,7 +217,7 @@ slr_status upload_operator(slr_handle h, DevOperator<T>& op, bool with_band) {
                 mx = std::max(mx, nJ * (nJ + 1) / 2 + nr * (nJ | 1));
             }
             d.lev_stage[l] = (int32_t)std::min(mx, capmax);
-            d.stage_cap = std::max(d.stage_cap, d.lev_stage[l]);
+            d.stage_cap = std::max(d.stage_cap, (int32_t)std::min<int64_t>(d.lev_stage[l], perscap));
         }
     }
     CS(dalloc(h, &d.bar, 1));

@@ -206,46 +206,7 @@ __device__ __forceinline__ T t_entry(const CView<T>& cf, int32_t pos, const T* g
            gather_sum(cf.wbuf + j, cf.wr, cf.seg_row, cf.seg_ptr[pos], cf.seg_ptr[pos + 1]);
 }
 
-// t at position pos for right-hand sides j .. j + nb - 1 (nb <= 8) into out[0 .. 8)
-// (zeros past nb): the index chain is loaded once for the eight, each sum still
-// takes its contributions in order, as t_entry does
-template <typename T>
-__device__ __forceinline__ void t_entry8(const CView<T>& cf, int32_t pos, const T* g, int64_t ldg, int j, int nb,
-                                         T (&out)[8]) {
-    const int64_t e0 = cf.seg_ptr[pos], e1 = cf.seg_ptr[pos + 1];
-    T acc[8];
-#pragma unroll
-    for (int b = 0; b < 8; ++b) acc[b] = T(0);
-    for (int64_t e = e0; e < e1; e += 4) {
-        int32_t idx[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) idx[u] = e + u < e1 ? cf.seg_row[e + u] : -1;
-        T v[4][8];
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-#pragma unroll
-            for (int b = 0; b < 8; ++b)
-                v[u][b] = (idx[u] >= 0 && b < nb) ? cf.wbuf[(int64_t)idx[u] * cf.wr + j + b] : T(0);
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (idx[u] >= 0) {
-#pragma unroll
-                for (int b = 0; b < 8; ++b) acc[b] += v[u][b];
-            }
-    }
-#pragma unroll
-    for (int b = 0; b < 8; ++b) out[b] = b < nb ? g_at(cf, pos, g, ldg, j + b) - acc[b] : T(0);
-}
-
-// t_J = g_J - gathered panel products into ts[0 .. n_J) by NTH threads (thread gt)
-template <typename T>
-__device__ __forceinline__ void gather_t(const CView<T>& cf, int J, int gt, int nth, T* ts, const T* g, int64_t ldg,
-                                         int j) {
-    const int32_t a0 = cf.c0[J], nJ = cf.c0[J + 1] - a0;
-    for (int i = gt; i < nJ; i += nth) ts[i] = t_entry(cf, a0 + i, g, ldg, j);
-}
-
-// eight consecutive values from shared memory (p 16-byte aligned)
+// eight consecutive values (p 16-byte aligned)
 template <typename T>
 __device__ __forceinline__ void ld8(const T* p, T (&v)[8]) {
     if constexpr (sizeof(T) == 4) {
@@ -261,6 +222,90 @@ __device__ __forceinline__ void ld8(const T* p, T (&v)[8]) {
         }
     }
 }
+
+// elements of a 16-byte word
+template <typename T>
+__host__ __device__ constexpr int vec_elems() { return 16 / (int)sizeof(T); }
+// rows of ld elements at p all start on 16-byte boundaries
+template <typename T>
+__device__ __forceinline__ bool rows_vec(const T* p, int64_t ld) {
+    return ld % vec_elems<T>() == 0 && reinterpret_cast<uintptr_t>(p) % 16 == 0;
+}
+
+// v[0 .. nb) = p[0 .. nb), zeros past nb (nb <= 8); vec: p is 16-byte aligned
+template <typename T>
+__device__ __forceinline__ void load_row8(const T* p, int nb, bool vec, T (&v)[8]) {
+    if (vec && nb >= 8) {
+        ld8(p, v);
+    } else {
+#pragma unroll
+        for (int b = 0; b < 8; ++b) v[b] = b < nb ? p[b] : T(0);
+    }
+}
+// p[0 .. nb) = v[0 .. nb) (nb <= 8); vec: p is 16-byte aligned
+template <typename T>
+__device__ __forceinline__ void store_row8(T* p, int nb, bool vec, const T (&v)[8]) {
+    if (vec && nb >= 8) {
+        if constexpr (sizeof(T) == 4) {
+            reinterpret_cast<float4*>(p)[0] = make_float4(v[0], v[1], v[2], v[3]);
+            reinterpret_cast<float4*>(p)[1] = make_float4(v[4], v[5], v[6], v[7]);
+        } else {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) reinterpret_cast<double2*>(p)[q] = make_double2(v[2 * q], v[2 * q + 1]);
+        }
+    } else {
+#pragma unroll
+        for (int b = 0; b < 8; ++b)
+            if (b < nb) p[b] = v[b];
+    }
+}
+
+// t at position pos for right-hand sides j .. j + nb - 1 (nb <= 8) into out[0 .. 8)
+// (zeros past nb): the index chain is loaded once for the eight, each sum still
+// takes its contributions in order, as t_entry does.  vec: rows of w and of g (in factor order)
+// start on 16-byte boundaries and j is a multiple of 8, so a row's eight are two words.
+template <typename T>
+__device__ __forceinline__ void t_entry8(const CView<T>& cf, int32_t pos, const T* g, int64_t ldg, int j, int nb,
+                                         bool vec, T (&out)[8]) {
+    const int64_t e0 = cf.seg_ptr[pos], e1 = cf.seg_ptr[pos + 1];
+    T acc[8], gv[8];
+    if (cf.gf) {
+        load_row8(cf.gf + (int64_t)pos * cf.wr + j, nb, vec, gv);
+    } else {
+        const int64_t gi = cf.cperm[pos];
+#pragma unroll
+        for (int b = 0; b < 8; ++b) gv[b] = b < nb ? g[gi + (int64_t)(j + b) * ldg] : T(0);
+    }
+#pragma unroll
+    for (int b = 0; b < 8; ++b) acc[b] = T(0);
+    constexpr int EB = 2;                              // rows in flight (four spill)
+    for (int64_t e = e0; e < e1; e += EB) {
+        int32_t idx[EB];
+#pragma unroll
+        for (int u = 0; u < EB; ++u) idx[u] = e + u < e1 ? cf.seg_row[e + u] : -1;
+        T v[EB][8];
+#pragma unroll
+        for (int u = 0; u < EB; ++u)
+            if (idx[u] >= 0) load_row8(cf.wbuf + (int64_t)idx[u] * cf.wr + j, nb, vec, v[u]);
+#pragma unroll
+        for (int u = 0; u < EB; ++u)
+            if (idx[u] >= 0) {
+#pragma unroll
+                for (int b = 0; b < 8; ++b) acc[b] += v[u][b];
+            }
+    }
+#pragma unroll
+    for (int b = 0; b < 8; ++b) out[b] = b < nb ? gv[b] - acc[b] : T(0);
+}
+
+// t_J = g_J - gathered panel products into ts[0 .. n_J) by NTH threads (thread gt)
+template <typename T>
+__device__ __forceinline__ void gather_t(const CView<T>& cf, int J, int gt, int nth, T* ts, const T* g, int64_t ldg,
+                                         int j) {
+    const int32_t a0 = cf.c0[J], nJ = cf.c0[J + 1] - a0;
+    for (int i = gt; i < nJ; i += nth) ts[i] = t_entry(cf, a0 + i, g, ldg, j);
+}
+
 // right-hand sides per pass of the tiled small-supernode paths
 template <typename T>
 __host__ __device__ constexpr int tile_rp() { return sizeof(T) == 4 ? 32 : 16; }
@@ -869,104 +914,124 @@ __device__ __forceinline__ bool stage_block_fwd(const CView<T>& cf, int J, T* st
 // virtual rows; a warp takes 128 of them (lane + 32 u, u < 4) for 8 right-hand
 // sides, so that each thread holds 4 x 8 sums and a column costs four matrix loads
 // and two 16-byte loads of t_J (stored right-hand sides contiguous, RP per pass)
-// for 32 multiply-adds.  Each (row, right-hand side) still takes its multiply-adds
+// for 32 multiply-adds; 64 or 32 of them where 128 would leave warps without a tile (a leaf
+// of 3-D 96^3 has about 90 rows: with 32 right-hand sides, four tiles of 128 for eight warps).  Each (row, right-hand side) still takes its multiply-adds
 // over the columns in order from zero; a diagonal row adds exact zeros past its
 // last column, so the bits are those of the row-per-thread path.
+template <typename T, int U>
+__device__ __forceinline__ void cfwd_tile(const CView<T>& cf, int32_t a0, int32_t nJ, int32_t nr, const T* ts, int RP,
+                                          int rbase, int h, int j0, int nb, T* xf, T* wb, bool vec, const T* D,
+                                          const T* Pn) {
+    const int lane = threadIdx.x & 31;
+    const int32_t ND = (nJ + 31) & ~31, RV = ND + nr, ldp = small_ldp(nJ);
+    int kind[U], r[U], cend = 0;           // kind (warp-uniform): 0 none, 1 diagonal, 2 panel
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const int v0 = rbase + 32 * u;
+        kind[u] = v0 < ND ? 1 : (v0 < RV ? 2 : 0);
+        r[u] = v0 + lane;
+        if (kind[u] == 1) cend = max(cend, min(nJ, v0 + 32));
+        if (kind[u] == 2) cend = nJ;
+    }
+    T acc[U][8];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int b = 0; b < 8; ++b) acc[u][b] = T(0);
+    int32_t pcm = 0;                       // packed_col(c) - c
+    for (int c = 0; c < cend; ++c) {
+        T tv[8];
+        ld8(ts + c * RP + 8 * h, tv);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (kind[u] == 0) continue;
+            T a = T(0);
+            if (kind[u] == 1) {
+                if (r[u] >= c && r[u] < nJ) a = D[pcm + r[u]];
+            } else if (r[u] < RV) {
+                a = Pn[(r[u] - ND) * ldp + c];
+            }
+#pragma unroll
+            for (int b = 0; b < 8; ++b) acc[u][b] = fma(a, tv[b], acc[u][b]);
+        }
+        pcm += nJ - c - 1;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        if (kind[u] == 1 && r[u] < nJ) {
+#pragma unroll
+            for (int b = 0; b < 8; ++b)
+                if (8 * h + b < nb) xf[a0 + r[u] + (int64_t)(j0 + 8 * h + b) * cf.s] = acc[u][b];
+        } else if (kind[u] == 2 && r[u] < RV) {
+            store_row8(wb + (int64_t)(r[u] - ND) * cf.wr + j0 + 8 * h, nb - 8 * h, vec, acc[u]);
+        }
+    }
+}
+
 template <typename T, int NT, int GROUPS>
 __device__ void cfwd_small_tiled(const CView<T>& cf, int J, T* ts, const T* g, int64_t ldg, T* xf, int32_t nrhs,
                                  const T* D, const T* Pn) {
     constexpr int nw = NT / 32, RPM = tile_rp<T>();
-    const int gt = threadIdx.x % NT, lane = gt & 31, warp = gt >> 5;
+    const int gt = threadIdx.x % NT, warp = gt >> 5;
     const int32_t a0 = cf.c0[J], nJ = cf.c0[J + 1] - a0;
     const int32_t nr = (int32_t)(cf.r_off[J + 1] - cf.r_off[J]);
-    const int32_t ND = (nJ + 31) & ~31, RV = ND + nr, ldp = small_ldp(nJ);
+    const int32_t RV = ((nJ + 31) & ~31) + nr;
     T* wb = cf.wbuf + cf.r_off[J] * cf.wr;
+    const bool vec = rows_vec(cf.wbuf, cf.wr) && rows_vec(cf.gf, cf.wr);
     for (int j0 = 0; j0 < nrhs; j0 += RPM) {
         const int nb = min(RPM, nrhs - j0), RP = (nb + 7) & ~7, ngrp = RP / 8;
         for (int it = gt; it < nJ * ngrp; it += NT) {
             const int i = it / ngrp, h = it - i * ngrp;
             T tv[8];
-            t_entry8(cf, a0 + i, g, ldg, j0 + 8 * h, nb - 8 * h, tv);
-#pragma unroll
-            for (int b = 0; b < 8; ++b) ts[i * RP + 8 * h + b] = tv[b];
+            t_entry8(cf, a0 + i, g, ldg, j0 + 8 * h, nb - 8 * h, vec, tv);
+            store_row8(ts + i * RP + 8 * h, 8, true, tv);
         }
         if (j0 == 0) stage_wait();
         group_sync<NT, GROUPS>();
-        const int items = ((RV + 127) >> 7) * ngrp;
-        for (int it = warp; it < items; it += nw) {
-            const int tile = it / ngrp, h = it - tile * ngrp, rbase = tile * 128;
-            int kind[4], r[4], cend = 0;       // kind (warp-uniform): 0 none, 1 diagonal, 2 panel
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int v0 = rbase + 32 * u;
-                kind[u] = v0 < ND ? 1 : (v0 < RV ? 2 : 0);
-                r[u] = v0 + lane;
-                if (kind[u] == 1) cend = max(cend, min(nJ, v0 + 32));
-                if (kind[u] == 2) cend = nJ;
-            }
-            T acc[4][8];
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int b = 0; b < 8; ++b) acc[u][b] = T(0);
-            int32_t pcm = 0;                   // packed_col(c) - c
-            for (int c = 0; c < cend; ++c) {
-                T tv[8];
-                ld8(ts + c * RP + 8 * h, tv);
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    if (kind[u] == 0) continue;
-                    T a = T(0);
-                    if (kind[u] == 1) {
-                        if (r[u] >= c && r[u] < nJ) a = D[pcm + r[u]];
-                    } else if (r[u] < RV) {
-                        a = Pn[(r[u] - ND) * ldp + c];
-                    }
-#pragma unroll
-                    for (int b = 0; b < 8; ++b) acc[u][b] = fma(a, tv[b], acc[u][b]);
-                }
-                pcm += nJ - c - 1;
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int b = 0; b < 8; ++b) {
-                    const int j = 8 * h + b;
-                    if (j >= nb) continue;
-                    if (kind[u] == 1 && r[u] < nJ) xf[a0 + r[u] + (int64_t)(j0 + j) * cf.s] = acc[u][b];
-                    else if (kind[u] == 2 && r[u] < RV) wb[(int64_t)(r[u] - ND) * cf.wr + j0 + j] = acc[u][b];
-                }
+        const int t4 = ((RV + 127) >> 7) * ngrp, t2 = ((RV + 63) >> 6) * ngrp;
+        if (sizeof(T) == 4 && t4 >= nw) {
+            if constexpr (sizeof(T) == 4)              // FP64: its pipe sets the pace, and 4 x 8 sums spill
+                for (int it = warp; it < t4; it += nw)
+                    cfwd_tile<T, 4>(cf, a0, nJ, nr, ts, RP, (it / ngrp) * 128, it % ngrp, j0, nb, xf, wb, vec, D, Pn);
+        } else if (t2 >= nw) {
+            for (int it = warp; it < t2; it += nw)
+                cfwd_tile<T, 2>(cf, a0, nJ, nr, ts, RP, (it / ngrp) * 64, it % ngrp, j0, nb, xf, wb, vec, D, Pn);
+        } else {
+            const int t1 = ((RV + 31) >> 5) * ngrp;
+            for (int it = warp; it < t1; it += nw)
+                cfwd_tile<T, 1>(cf, a0, nJ, nr, ts, RP, (it / ngrp) * 32, it % ngrp, j0, nb, xf, wb, vec, D, Pn);
         }
         group_sync<NT, GROUPS>();
     }
 }
 
-template <typename T, int NT, int GROUPS, int RB>
+template <typename T, int NT, int GROUPS, int RB, bool TILED = false>
 __device__ void cfwd_small_cta(const CView<T>& cf, int J, T* ts, const T* g, int64_t ldg, T* xf, int32_t nrhs, T* stg,
-                               int cap, bool tiled = false) {
+                               int cap) {
     constexpr int nw = NT / 32;
     const int gt = threadIdx.x % NT, lane = gt & 31, warp = gt >> 5;
     const int32_t a0 = cf.c0[J], nJ = cf.c0[J + 1] - a0;
     const int64_t nr = cf.r_off[J + 1] - cf.r_off[J], rtot = nJ + nr;
     const T *D, *Pn;
     const bool staged = stage_block_fwd<T, NT>(cf, J, stg, cap, gt, D, Pn);   // lands while t_J is gathered
-    if (tiled && staged) {
-        cfwd_small_tiled<T, NT, GROUPS>(cf, J, ts, g, ldg, xf, nrhs, D, Pn);
-        return;
-    }
-    if (tiled) {
+    if constexpr (TILED) {
+        if (staged) {
+            cfwd_small_tiled<T, NT, GROUPS>(cf, J, ts, g, ldg, xf, nrhs, D, Pn);
+            return;
+        }
         // Blocks of 8 or more on a block left in HBM: t_J of up to tile_rp<T>() columns
         // gathered at once (column-major, kSmallN apart: ts holds kSmallN x tile_rp), then
         // the warp-per-four-rows products of the path below for each group of 8 columns,
         // whose 32 warp sums per quad of rows are formed by one reduce-scatter (warp_sum's
         // tree, bit for bit); the block is re-read from cache for each group.
         constexpr int RPM = tile_rp<T>();
+        const bool vec = rows_vec(cf.wbuf, cf.wr) && rows_vec(cf.gf, cf.wr);
         for (int j0 = 0; j0 < nrhs; j0 += RPM) {
             const int nbp = min(RPM, nrhs - j0);
             for (int it = gt; it < nJ * ((nbp + 7) / 8); it += NT) {
                 const int i = it % nJ, h = it / nJ;
                 T tv[8];
-                t_entry8(cf, a0 + i, g, ldg, j0 + 8 * h, nbp - 8 * h, tv);
+                t_entry8(cf, a0 + i, g, ldg, j0 + 8 * h, nbp - 8 * h, vec, tv);
 #pragma unroll
                 for (int b = 0; b < 8; ++b) ts[(8 * h + b) * kSmallN + i] = tv[b];
             }
@@ -1104,6 +1169,7 @@ __device__ void cbwd_small_tiled(const CView<T>& cf, int J, T* vs, const T* yf, 
     while (P < nJ) P *= 2;
     const int parts = NT / P, ncg = (nJ + 3) / 4;
     const int64_t len = (rtot + parts - 1) / parts;
+    const bool vec = rows_vec<T>(xf, cf.xr);
     int32_t pcm[4];                                      // packed_col(c) - c of the thread's columns
     for (int j0 = 0; j0 < nrhs; j0 += rpm) {
         const int nb = min(rpm, nrhs - j0), RP = (nb + 7) & ~7, ngrp = RP / 8;
@@ -1111,16 +1177,17 @@ __device__ void cbwd_small_tiled(const CView<T>& cf, int J, T* vs, const T* yf, 
         for (int64_t it = gt; it < rtot * ngrp; it += NT) {
             const int64_t r = it / ngrp;
             const int h = (int)(it - r * ngrp);
-            const int64_t src = r < nJ ? a0 + r : R[r - nJ];
             T v[8];
+            if (r < nJ) {
 #pragma unroll
-            for (int b = 0; b < 8; ++b) {
-                const int j = 8 * h + b;
-                v[b] = T(0);
-                if (j < nb) v[b] = r < nJ ? yf[src + (int64_t)(j0 + j) * cf.s] : -xf[src * cf.xr + j0 + j];
+                for (int b = 0; b < 8; ++b)
+                    v[b] = 8 * h + b < nb ? yf[a0 + r + (int64_t)(j0 + 8 * h + b) * cf.s] : T(0);
+            } else {
+                load_row8<T>(xf + (int64_t)R[r - nJ] * cf.xr + j0 + 8 * h, nb - 8 * h, vec, v);
+#pragma unroll
+                for (int b = 0; b < 8; ++b) v[b] = 8 * h + b < nb ? -v[b] : T(0);
             }
-#pragma unroll
-            for (int b = 0; b < 8; ++b) vs[r * RP + 8 * h + b] = v[b];
+            store_row8(vs + r * RP + 8 * h, 8, true, v);
         }
         if (j0 == 0) stage_wait();
         group_sync<NT, GROUPS>();
@@ -1160,11 +1227,7 @@ __device__ void cbwd_small_tiled(const CView<T>& cf, int J, T* vs, const T* yf, 
         if (act) {
 #pragma unroll
             for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int b = 0; b < 8; ++b) {
-                    const int c = 4 * cg + i, j = 8 * h + b;
-                    if (c < nJ && j < nb) vs[((int64_t)q * nJ + c) * RP + j] = acc[i][b];
-                }
+                if (4 * cg + i < nJ) store_row8(vs + ((int64_t)q * nJ + 4 * cg + i) * RP + 8 * h, 8, true, acc[i]);
         }
         group_sync<NT, GROUPS>();
         for (int idx = gt; idx < nJ * nb; idx += NT) {
@@ -1178,9 +1241,9 @@ __device__ void cbwd_small_tiled(const CView<T>& cf, int J, T* vs, const T* yf, 
     }
 }
 
-template <typename T, int NT, int GROUPS, int RB>
+template <typename T, int NT, int GROUPS, int RB, bool TILED = false>
 __device__ void cbwd_small_cta(const CView<T>& cf, int J, T* vs, T* red, const T* yf, T* xf, T* y_dd, int64_t ldy,
-                               int32_t nrhs, T* stg, int cap, bool tiled = false) {
+                               int32_t nrhs, T* stg, int cap) {
     static_assert(NT % kSmallN == 0 && NT <= 1024, "whole parts per column");
     constexpr int VS = kSmallN + kSmallR;
     const int gt = threadIdx.x % NT;
@@ -1189,7 +1252,7 @@ __device__ void cbwd_small_cta(const CView<T>& cf, int J, T* vs, T* red, const T
     const int32_t* R = cf.rows + cf.r_off[J];
     const T *D, *Pn;
     const bool staged = stage_block<T, NT>(cf, J, stg, cap, gt, D, Pn);   // lands while the vector is staged
-    if (tiled) {
+    if constexpr (TILED) {
         // right-hand sides per pass: the vector (rows x RP) and the sums (NT x RP) fit the buffer
         const int rpm = min(tile_rp<T>(), (int)(tile_vs<T>() / max(rtot, (int64_t)NT)) & ~7);
         if (rpm >= 8) {
@@ -1321,6 +1384,27 @@ k_cperm_g(int32_t s, int32_t nrhs, const int32_t* __restrict__ ciperm, const T* 
     }
 }
 
+// y[i + j ldy] = xf[ciperm[i] nrhs + j]: the backward's solution in DD order.  The level kernels
+// scattered each value of a block as they formed it, a 32-byte sector per 4-byte value; a
+// row of xf is read as whole lines here, and y written along i.
+template <typename T>
+__global__ void __launch_bounds__(256)
+k_cperm_y(int32_t s, int32_t nrhs, const int32_t* __restrict__ ciperm, const T* __restrict__ xf, T* y, int64_t ldy) {
+    __shared__ T tile[32][33];
+    const int i0 = blockIdx.x * 32, j0 = blockIdx.y * 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int il = ty + 8 * q, i = i0 + il, j = j0 + tx;
+        if (i < s && j < nrhs) tile[il][tx] = xf[(int64_t)ciperm[i] * nrhs + j];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int i = i0 + tx, j = j0 + ty + 8 * q;
+        if (i < s && j < nrhs) y[i + (int64_t)j * ldy] = tile[tx][ty + 8 * q];
+    }
+}
+
 // t_J = g_J - (gathered panel products) for every supernode of a level, once, into
 // cf.tws: block (q, c) takes entries c * 256 .. c * 256 + 255 of the (position,
 // right-hand side) pairs of the level's q-th supernode.  The per-level forward tasks
@@ -1374,50 +1458,48 @@ k_cbwd_level_blk(const CView<T> cf, int32_t t0, const T* yf, T* xf, T* y_dd, int
 // tiled paths.
 // dynamic shared memory: t_J (tsz elements: RB right-hand sides, or tile_rp
 // contiguous ones for the tiled path), then the stage buffer of cap elements
-template <typename T, int RB>
+template <typename T, int RB, bool TILED>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 2)
-k_cfwd_small(const CView<T> cf, int32_t s0, const T* g, int64_t ldg, T* xf, int32_t nrhs, int32_t cap, int32_t tsz,
-             bool tiled) {
+k_cfwd_small(const CView<T> cf, int32_t s0, const T* g, int64_t ldg, T* xf, int32_t nrhs, int32_t cap,
+             int32_t tsz) {
     extern __shared__ __align__(16) unsigned char csm[];
     T* ts = reinterpret_cast<T*>(csm);
-    cfwd_small_cta<T, kThreads, 1, RB>(cf, cf.lev_sn[s0 + blockIdx.x], ts, g, ldg, xf, nrhs, ts + tsz, cap, tiled);
+    cfwd_small_cta<T, kThreads, 1, RB, TILED>(cf, cf.lev_sn[s0 + blockIdx.x], ts, g, ldg, xf, nrhs, ts + tsz, cap);
 }
 
 // dynamic shared memory (vsz elements): RB vectors of kSmallN + kSmallR and
 // RB x kThreads partial sums, or for blocks of 8 or more the tiled path's
 // buffer if that is more, then the stage buffer of cap elements
-template <typename T, int RB>
+template <typename T, int RB, bool TILED>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 2)
 k_cbwd_small(const CView<T> cf, int32_t s0, const T* yf, T* xf, T* y_dd, int64_t ldy, int32_t nrhs, int32_t cap,
-             int32_t vsz, bool tiled) {
+             int32_t vsz) {
     extern __shared__ __align__(16) unsigned char csm[];
     T* vs = reinterpret_cast<T*>(csm);
     T* red = vs + RB * (kSmallN + kSmallR);
-    cbwd_small_cta<T, kThreads, 1, RB>(cf, cf.lev_sn[s0 + blockIdx.x], vs, red, yf, xf, y_dd, ldy, nrhs, vs + vsz, cap,
-                                       tiled);
+    cbwd_small_cta<T, kThreads, 1, RB, TILED>(cf, cf.lev_sn[s0 + blockIdx.x], vs, red, yf, xf, y_dd, ldy, nrhs, vs + vsz,
+                                              cap);
 }
 
-template <typename T, int RB>
+template <typename T, int RB, bool TILED = false>
 cudaError_t cfwd_small_launch(const CView<T>& v, int s0, int ns, int32_t cap, const T* g, int64_t ldg, T* xf,
                               int32_t nrhs, cudaStream_t st) {
-    const bool tiled = nrhs >= 8;
-    const int32_t tsz = tiled ? kSmallN * tile_rp<T>() : RB * kSmallN;
+    const int32_t tsz = TILED ? kSmallN * tile_rp<T>() : RB * kSmallN;
     const size_t sm = ((size_t)tsz + cap) * sizeof(T);
-    auto kern = k_cfwd_small<T, RB>;
+    auto kern = k_cfwd_small<T, RB, TILED>;
     if (sm > 48 * 1024 && !raise_smem_once((const void*)kern)) return cudaErrorInvalidValue;
-    kern<<<ns, kThreads, sm, st>>>(v, s0, g, ldg, xf, nrhs, cap, tsz, tiled);
+    kern<<<ns, kThreads, sm, st>>>(v, s0, g, ldg, xf, nrhs, cap, tsz);
     count_launches(1);
     return cudaGetLastError();
 }
-template <typename T, int RB>
+template <typename T, int RB, bool TILED = false>
 cudaError_t cbwd_small_launch(const CView<T>& v, int s0, int ns, int32_t cap, const T* yf, T* xf, T* y_dd, int64_t ldy,
                               int32_t nrhs, cudaStream_t st) {
-    const bool tiled = nrhs >= 8;
-    const int32_t plain = RB * (kSmallN + kSmallR + kThreads), vsz = tiled ? std::max(tile_vs<T>(), plain) : plain;
+    const int32_t plain = RB * (kSmallN + kSmallR + kThreads), vsz = TILED ? std::max(tile_vs<T>(), plain) : plain;
     const size_t sm = ((size_t)vsz + cap) * sizeof(T);
-    auto kern = k_cbwd_small<T, RB>;
+    auto kern = k_cbwd_small<T, RB, TILED>;
     if (sm > 48 * 1024 && !raise_smem_once((const void*)kern)) return cudaErrorInvalidValue;
-    kern<<<ns, kThreads, sm, st>>>(v, s0, yf, xf, y_dd, ldy, nrhs, cap, vsz, tiled);
+    kern<<<ns, kThreads, sm, st>>>(v, s0, yf, xf, y_dd, ldy, nrhs, cap, vsz);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -2264,7 +2346,8 @@ cudaError_t launch_c_forward(const DevCFactor<T>& cf, const T* g_dd, int64_t ldg
                 nrhs == 1   ? cfwd_small_launch<T, 1>(v, s0, ns, cap, g_dd, ldg, xf, nrhs, st)
                 : nrhs == 2 ? cfwd_small_launch<T, 2>(v, s0, ns, cap, g_dd, ldg, xf, nrhs, st)
                 : nrhs <= 4 ? cfwd_small_launch<T, 4>(v, s0, ns, cap, g_dd, ldg, xf, nrhs, st)
-                            : cfwd_small_launch<T, 8>(v, s0, ns, cap, g_dd, ldg, xf, nrhs, st);
+                : nrhs < 8  ? cfwd_small_launch<T, 8>(v, s0, ns, cap, g_dd, ldg, xf, nrhs, st)
+                            : cfwd_small_launch<T, 8, true>(v, s0, ns, cap, g_dd, ldg, xf, nrhs, st);
             if (e != cudaSuccess) return e;
             continue;
         }
@@ -2333,8 +2416,8 @@ cudaError_t launch_c_forward(const DevCFactor<T>& cf, const T* g_dd, int64_t ldg
 }
 
 template <typename T>
-cudaError_t launch_c_backward(const DevCFactor<T>& cf, const T* yf, T* xf, T* y_dd, int64_t ldy, int32_t nrhs,
-                              cudaStream_t st) {
+cudaError_t c_backward_steps(const DevCFactor<T>& cf, const T* yf, T* xf, T* y_dd, int64_t ldy, int32_t nrhs,
+                             cudaStream_t st) {
     if (cf.nT > 0 && nrhs > cf.ws_cols) return cudaErrorInvalidValue;
     CView<T> v = make_view(cf, cf.nsteps_bwd);
     v.xr = nrhs;     // the solution x (scratch): a call's right-hand sides contiguous per row
@@ -2360,7 +2443,8 @@ cudaError_t launch_c_backward(const DevCFactor<T>& cf, const T* yf, T* xf, T* y_
             const cudaError_t e =
                 nrhs == 1   ? cbwd_small_launch<T, 1>(v, s0, ns, cap, yf, xf, y_dd, ldy, nrhs, st)
                 : nrhs == 2 ? cbwd_small_launch<T, 2>(v, s0, ns, cap, yf, xf, y_dd, ldy, nrhs, st)
-                            : cbwd_small_launch<T, 4>(v, s0, ns, cap, yf, xf, y_dd, ldy, nrhs, st);
+                : nrhs < 8  ? cbwd_small_launch<T, 4>(v, s0, ns, cap, yf, xf, y_dd, ldy, nrhs, st)
+                            : cbwd_small_launch<T, 4, true>(v, s0, ns, cap, yf, xf, y_dd, ldy, nrhs, st);
             if (e != cudaSuccess) return e;
             continue;
         }
@@ -2400,6 +2484,20 @@ cudaError_t launch_c_backward(const DevCFactor<T>& cf, const T* yf, T* xf, T* y_
         }
         counted();
     }
+    return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_c_backward(const DevCFactor<T>& cf, const T* yf, T* xf, T* y_dd, int64_t ldy, int32_t nrhs,
+                              cudaStream_t st) {
+    // large blocks: the solution stays in xf until every row is there, then goes to DD order at once
+    // (3-D 96^3 with 32 columns, s = 249k: apply 2784 -> 2758 us; s = 15k with 8 columns: the
+    // launch costs 3 us more than the scatter, so small calls scatter)
+    const bool after = nrhs >= 8 && (int64_t)cf.s * nrhs >= 1 << 20 && y_dd && cf.ciperm;
+    const cudaError_t e = c_backward_steps<T>(cf, yf, xf, after ? nullptr : y_dd, ldy, nrhs, st);
+    if (e != cudaSuccess || !after) return e;
+    k_cperm_y<T><<<dim3((cf.s + 31) / 32, (nrhs + 31) / 32), 256, 0, st>>>(cf.s, nrhs, cf.ciperm, xf, y_dd, ldy);
+    counted();
     return cudaGetLastError();
 }
 
