@@ -1154,10 +1154,58 @@ __host__ __device__ constexpr int tile_vs() { return sizeof(T) == 4 ? 8192 : 409
 // Blocks of right-hand sides (tiled backward): the rows of A_J split into the same
 // parts as the column-per-thread path below, and a thread takes 4 columns x 8
 // right-hand sides of one part (a row costs four matrix loads and two 16-byte loads
-// of the stacked vector, stored right-hand sides contiguous, for 32 multiply-adds).
+// of the stacked vector, stored right-hand sides contiguous, for 32 multiply-adds), or
+// fewer columns where four would leave threads idle (16 right-hand sides on a leaf of 20 columns:
+// 80 of 256 threads, and half the stalls at the barrier behind them).
 // Each (column, part) sums its rows in order from zero (diagonal rows above the
 // column add exact zeros) and the parts are added in order, as there: the same bits.
 // The vector buffer (rows x RP) then holds the parts' sums (at most NT x RP).
+// The products of one pass: a thread sums CT columns x 8 right-hand sides of one part, then, the
+// vector being read by all, leaves its sums in the vector's buffer.
+template <typename T, int NT, int GROUPS, int CT>
+__device__ __forceinline__ void cbwd_tile(int32_t nJ, int64_t rtot, int parts, int64_t len, int RP, int ngrp, T* vs,
+                                          const T* D, const T* Pn) {
+    const int gt = threadIdx.x % NT, ncg = (nJ + CT - 1) / CT;
+    const bool act = gt < parts * ngrp * ncg;          // at most NT items: one per thread
+    const int cg = act ? gt % ncg : 0, h = act ? (gt / ncg) % ngrp : 0, q = act ? gt / (ncg * ngrp) : 0;
+    T acc[CT][8];
+    int32_t pcm[CT];                                   // packed_col(c) - c of the thread's columns
+#pragma unroll
+    for (int i = 0; i < CT; ++i) {
+#pragma unroll
+        for (int b = 0; b < 8; ++b) acc[i][b] = T(0);
+        const int c = CT * cg + i;
+        pcm[i] = (int32_t)(packed_col(c, nJ) - c);
+    }
+    if (act) {
+        const int rb = (int)(q * len), re = (int)min(rtot, rb + len);
+        for (int r = rb; r < re; ++r) {
+            T tv[8];
+            ld8(vs + r * RP + 8 * h, tv);
+            T a[CT];
+#pragma unroll
+            for (int i = 0; i < CT; ++i) {
+                const int c = CT * cg + i;
+                a[i] = T(0);
+                if (c < nJ) {
+                    if (r >= nJ) a[i] = Pn[(r - nJ) * nJ + c];
+                    else if (r >= c) a[i] = D[pcm[i] + r];
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < CT; ++i)
+#pragma unroll
+                for (int b = 0; b < 8; ++b) acc[i][b] = fma(a[i], tv[b], acc[i][b]);
+        }
+    }
+    group_sync<NT, GROUPS>();                          // the vector is read: its buffer takes the sums
+    if (act) {
+#pragma unroll
+        for (int i = 0; i < CT; ++i)
+            if (CT * cg + i < nJ) store_row8(vs + (q * nJ + CT * cg + i) * RP + 8 * h, 8, true, acc[i]);
+    }
+}
+
 template <typename T, int NT, int GROUPS>
 __device__ void cbwd_small_tiled(const CView<T>& cf, int J, T* vs, const T* yf, T* xf, T* y_dd, int64_t ldy,
                                  int32_t nrhs, const T* D, const T* Pn, int rpm) {
@@ -1167,10 +1215,9 @@ __device__ void cbwd_small_tiled(const CView<T>& cf, int J, T* vs, const T* yf, 
     const int32_t* R = cf.rows + cf.r_off[J];
     int P = 32;
     while (P < nJ) P *= 2;
-    const int parts = NT / P, ncg = (nJ + 3) / 4;
+    const int parts = NT / P;
     const int64_t len = (rtot + parts - 1) / parts;
     const bool vec = rows_vec<T>(xf, cf.xr);
-    int32_t pcm[4];                                      // packed_col(c) - c of the thread's columns
     for (int j0 = 0; j0 < nrhs; j0 += rpm) {
         const int nb = min(rpm, nrhs - j0), RP = (nb + 7) & ~7, ngrp = RP / 8;
         // rows of [y_J; -x_{R_J}], eight right-hand sides per item (one index load)
@@ -1191,44 +1238,12 @@ __device__ void cbwd_small_tiled(const CView<T>& cf, int J, T* vs, const T* yf, 
         }
         if (j0 == 0) stage_wait();
         group_sync<NT, GROUPS>();
-        const int items = parts * ngrp * ncg;          // at most NT: one per thread
-        const bool act = gt < items;
-        const int cg = act ? gt % ncg : 0, h = act ? (gt / ncg) % ngrp : 0, q = act ? gt / (ncg * ngrp) : 0;
-        T acc[4][8];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-#pragma unroll
-            for (int b = 0; b < 8; ++b) acc[i][b] = T(0);
-            const int c = 4 * cg + i;
-            pcm[i] = (int32_t)(packed_col(c, nJ) - c);
-        }
-        if (act) {
-            const int64_t rb = q * len, re = min(rtot, rb + len);
-            for (int64_t r = rb; r < re; ++r) {
-                T tv[8];
-                ld8(vs + r * RP + 8 * h, tv);
-                T a[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int c = 4 * cg + i;
-                    a[i] = T(0);
-                    if (c < nJ) {
-                        if (r >= nJ) a[i] = Pn[(r - nJ) * nJ + c];
-                        else if (r >= c) a[i] = D[pcm[i] + r];
-                    }
-                }
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int b = 0; b < 8; ++b) acc[i][b] = fma(a[i], tv[b], acc[i][b]);
-            }
-        }
-        group_sync<NT, GROUPS>();                      // the vector is read: its buffer takes the sums
-        if (act) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-                if (4 * cg + i < nJ) store_row8(vs + ((int64_t)q * nJ + 4 * cg + i) * RP + 8 * h, 8, true, acc[i]);
-        }
+        // as few columns per thread as leave every item a thread
+        const int pg = parts * ngrp;
+        if (pg * nJ <= NT) cbwd_tile<T, NT, GROUPS, 1>(nJ, rtot, parts, len, RP, ngrp, vs, D, Pn);
+        else if (pg * ((nJ + 1) / 2) <= NT) cbwd_tile<T, NT, GROUPS, 2>(nJ, rtot, parts, len, RP, ngrp, vs, D, Pn);
+        else if (pg * ((nJ + 2) / 3) <= NT) cbwd_tile<T, NT, GROUPS, 3>(nJ, rtot, parts, len, RP, ngrp, vs, D, Pn);
+        else cbwd_tile<T, NT, GROUPS, 4>(nJ, rtot, parts, len, RP, ngrp, vs, D, Pn);
         group_sync<NT, GROUPS>();
         for (int idx = gt; idx < nJ * nb; idx += NT) {
             const int c = idx / nb, j = idx - c * nb;
