@@ -461,16 +461,35 @@ __device__ void cfwd_task_blk(const CView<T>& cf, const int4 tk, bool pan, T* ts
     const int ncl = pan ? nJ : tk.y + tk.z;        // columns the task reads
     const T* P = cf.panel + cf.pan_off[J];
     const int64_t w0 = cf.r_off[J];
-    for (int idx = threadIdx.x; idx < ncl * RP; idx += NW * 32) {
-        const int i = idx / RP, b = idx - i * RP;     // right-hand sides fastest: contiguous in the gather
-        ts[i * RS + b] = b < nb ? cf.tws[(int64_t)(a0 + i) * cf.wr + j0 + b] : T(0);
+    // the warp's first panel rows' first entries travel while t_J is staged
+    const T* Pp[R];
+    T an[R];
+    auto rows_at = [&](int pr) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            Pp[r] = P + (int64_t)(tk.y + min(pr + r, tk.z - 1)) * nJ;
+            an[r] = lane < nJ ? Pp[r][lane] : T(0);
+        }
+    };
+    if (pan) rows_at(warp * R);
+    if (rows_vec<T>(cf.tws, cf.wr) && nb == RP) {
+        constexpr int VE = vec_elems<T>(), NV = RP / VE;
+#pragma unroll 4
+        for (int idx = threadIdx.x; idx < ncl * NV; idx += NW * 32) {
+            const int i = idx / NV, b = (idx - i * NV) * VE;
+            *reinterpret_cast<uint4*>(ts + i * RS + b) =
+                *reinterpret_cast<const uint4*>(cf.tws + (int64_t)(a0 + i) * cf.wr + j0 + b);
+        }
+    } else {
+        for (int idx = threadIdx.x; idx < ncl * RP; idx += NW * 32) {
+            const int i = idx / RP, b = idx - i * RP;     // right-hand sides fastest: contiguous in the gather
+            ts[i * RS + b] = b < nb ? cf.tws[(int64_t)(a0 + i) * cf.wr + j0 + b] : T(0);
+        }
     }
     __syncthreads();
     if (pan) {
         for (int pr = warp * R; pr < tk.z; pr += NW * R) {
-            const T* Pp[R];
-#pragma unroll
-            for (int r = 0; r < R; ++r) Pp[r] = P + (int64_t)(tk.y + min(pr + r, tk.z - 1)) * nJ;
+            if (pr > warp * R) rows_at(pr);
             T acc[R][RP];
 #pragma unroll
             for (int r = 0; r < R; ++r)
@@ -488,11 +507,8 @@ __device__ void cfwd_task_blk(const CView<T>& cf, const int4 tk, bool pan, T* ts
                 }
             };
             // the next columns' entries are in flight during a step's products
-            T a[R], an[R];
-            int c = lane;
-#pragma unroll
-            for (int r = 0; r < R; ++r) an[r] = c < nJ ? Pp[r][c] : T(0);
-            for (; c < nJ; c += 32) {
+            T a[R];
+            for (int c = lane; c < nJ; c += 32) {
 #pragma unroll
                 for (int r = 0; r < R; ++r) a[r] = an[r];
                 if (c + 32 < nJ) {
@@ -663,8 +679,8 @@ __device__ void cbwd_task_rb(const CView<T>& cf, const int4 tk, T* us, T (*red)[
 // part with lanes over the columns and the warps splitting the panel rows, each warp
 // gathering 32 rows of x_{R_J} at a time into its own part of xs (row stride RP + 4)
 // and reading them back by 16-byte broadcasts.  A batch costs two latencies: its row
-// numbers are loaded during the batch before it, all its rows of x at once, and the
-// panel's entries eight rows ahead of their products.  The
+// numbers are loaded during the batch before it, all its rows of x at once (the first
+// batch's before the diagonal part), and the panel's entries eight rows ahead of their products.  The
 // partial sums then go to xs (the same buffer) and are added over the warps in
 // order.  Every column gets cbwd_task_rb's multiply-adds and additions, bit for bit.
 // us: RP x 32; xs: NW x 32 x (RP + 4).
@@ -682,6 +698,27 @@ __device__ void cbwd_task_blk(const CView<T>& cf, const int4 tk, T* us, T* xs, T
     const T* y = yf + a0 + (int64_t)j0 * cf.s;
     const T* x = xf + j0;                    // x(pos, b) at x[pos xr + b]
     int32_t rnext = pb + lane < pe ? R[pb + lane] : 0;
+    T* xw = xs + (size_t)warp * 32 * RS;               // this warp's rows
+    const int gb = lane % RP, gr = lane / RP;          // the right-hand side and row a lane gathers
+    // x_{R_J} rows q0 .. q0 + nq - 1 into xw; the next batch's row numbers on their way
+    auto gather_x = [&](int64_t q0, int nq) {
+        const int32_t r = rnext;
+        rnext = q0 + 32 + lane < pe ? R[q0 + 32 + lane] : 0;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            T v[16 / NG];
+#pragma unroll
+            for (int u = 0; u < 16 / NG; ++u) {
+                const int row = 16 * h + u * NG + gr;
+                const int32_t pos = __shfl_sync(0xffffffffu, r, row & 31);
+                v[u] = (row < nq && gb < nb && gr < NG) ? x[(int64_t)pos * cf.xr + gb] : T(0);
+            }
+#pragma unroll
+            for (int u = 0; u < 16 / NG; ++u)
+                if (gr < NG) xw[(16 * h + u * NG + gr) * RS + gb] = v[u];
+        }
+    };
+    if (pb < pe) gather_x(pb, (int)min((int64_t)32, pe - pb));
     if (ystage) {
         for (int b = warp; b < RP; b += NW)
             for (int i = tk.y + lane; i < nJ; i += 32)
@@ -731,30 +768,13 @@ __device__ void cbwd_task_blk(const CView<T>& cf, const int4 tk, T* us, T* xs, T
     T acc[RP];
 #pragma unroll
     for (int b = 0; b < RP; ++b) acc[b] = T(0);
-    T* xw = xs + (size_t)warp * 32 * RS;               // this warp's rows
-    const int gb = lane % RP, gr = lane / RP;          // the right-hand side and row a lane gathers
     for (int64_t q0 = pb; q0 < pe; q0 += 32) {
         const int nq = (int)min((int64_t)32, pe - q0);
         const T* Pq = Pn + q0 * nJ;
         T pv[8];
 #pragma unroll
         for (int u = 0; u < 8; ++u) pv[u] = u < nq ? Pq[(int64_t)u * nJ] : T(0);
-        // x_{R_J} rows q0 .. q0 + nq - 1
-        const int32_t r = rnext;
-        rnext = q0 + 32 + lane < pe ? R[q0 + 32 + lane] : 0;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            T v[16 / NG];
-#pragma unroll
-            for (int u = 0; u < 16 / NG; ++u) {
-                const int row = 16 * h + u * NG + gr;
-                const int32_t pos = __shfl_sync(0xffffffffu, r, row & 31);
-                v[u] = (row < nq && gb < nb && gr < NG) ? x[(int64_t)pos * cf.xr + gb] : T(0);
-            }
-#pragma unroll
-            for (int u = 0; u < 16 / NG; ++u)
-                if (gr < NG) xw[(16 * h + u * NG + gr) * RS + gb] = v[u];
-        }
+        if (q0 > pb) gather_x(q0, nq);                 // (the first batch is there)
         __syncwarp();
         for (int p0 = 0; p0 < nq; p0 += 8) {
             T pc[8];
