@@ -96,8 +96,9 @@ typedef struct {
                                right-hand sides, narrower blocks take the FP32 kernel).
                                Must be SLR_U_FP32 with SLR_PREC_FP64                       */
 
-    /* ---- execution choices: each gives the same preconditioner up to rounding; the
-       band_* fields, c_persistent, host_loop and autotune give bitwise the same result */
+    /* ---- execution choices: each gives the same preconditioner up to rounding; band_slots,
+       band_order and host_loop give bitwise the same result (band_split, band_threads and
+       c_persistent, which autotune picks too, set how some sums are split)              */
     int32_t band_split;     /* CTAs (a thread-block cluster) per subdomain in the band solve:
                                1, 2 or 4; 0 = automatic                                  */
     int32_t band_slots;     /* shared-memory buffers the band solve streams its factor

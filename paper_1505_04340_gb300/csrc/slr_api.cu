@@ -202,7 +202,9 @@ slr_status upload_operator(slr_handle h, DevOperator<T>& op, bool with_band) {
         d.max_cta_tasks = std::max(d.max_cta_tasks, nt + np);
     }
     // fused levels stage a supernode's [L_JJ^{-1}; M_J] in shared memory when it fits
-    // 36 KB (the rest of the 48 KB default holds the kernels' static arrays); the
+    // 56 KB (three CTAs per SM beside their vectors: with 36 KB, FP64 3-D 64^3 took 1014 us
+    // per apply, 996 now, the C solve of 16 columns on 75 x 70 x 81 641, 615 now), the persistent
+    // kernels, four groups to a CTA, 36 KB each; the
     // forward stages the panel with an odd row stride (n_J | 1), so sizes count it
     {
         const int64_t capmax = 56 * 1024 / (int64_t)sizeof(T), perscap = 36 * 1024 / (int64_t)sizeof(T);
@@ -382,8 +384,10 @@ slr_status run_apply(slr_handle h, DevOperator<T>& op, const T* r, int64_t ldr, 
     const HostSetup& hs = h->hs;
     const int32_t nI = hs.nI, s = hs.s;
     CK(launch_band_solve<T>(op, hs.p, hs.wmax, r, ldr, op.tB, nI, nullptr, 0, nrhs, st));   // t = B^{-1} f
+    const bool zform = op.Zdd && h->k > 0;
+    DepScope dep(st, !zform);                            // (with a second stream plain launches)
     CK(launch_gather_et<T>(op, s, r + nI, ldr, op.tB, nI, op.gp, s, nrhs, st));              // g' = g - E^T t
-    if (op.Zdd && h->k > 0) {
+    if (zform) {
         // Z-form (Proposition 4.3, Eq. 4.15): v = d o Z_k^T g' on the side stream while
         // y = C^{-1} g' runs, then y = (1-theta)^{-1} y + Z_k v
         CK(cudaEventRecord(h->ev_fork, st));
@@ -410,6 +414,7 @@ slr_status apply_any(slr_handle h, const double* r, int64_t ldr, double* z, int6
     DevOperator<float>& op = h->op32;
     const int64_t n = h->hs.n;
     CK(launch_convert<double, float>(n, nrhs, r, ldr, op.wr, n, st));
+    DepScope dep(st);
     CS(run_apply<float>(h, op, op.wr, n, op.wz, n, nrhs, st));
     CK(launch_convert<float, double>(n, nrhs, op.wz, n, z, ldz, st));
     return SLR_OK;
@@ -1434,6 +1439,7 @@ slr_status slr_bsolve(slr_handle h, const double* f, double* t, int32_t nrhs, in
     }
     DevOperator<float>& op = h->op32;
     CK(launch_convert<double, float>(nI, nrhs, f, ld, op.wr, nI, st));
+    DepScope dep(st);
     CK(launch_band_solve<float>(op, h->hs.p, h->hs.wmax, op.wr, nI, op.wz, nI, nullptr, 0, nrhs, st));
     CK(launch_convert<float, double>(nI, nrhs, op.wz, nI, t, ld, st));
     return SLR_OK;
@@ -1453,12 +1459,14 @@ static slr_status interface_solve(slr_handle h, const double* g, double* y, int3
     if (h->opts.precision == SLR_PREC_FP64) {
         DevOperator<double>& op = h->op64;
         CK(launch_c_forward<double>(op.cf, g, ld, op.wf, nrhs, st));
+        DepScope dep(st);
         if (lowrank) CK(launch_lowrank<double>(op, s, h->k, op.wf, nrhs, st));
         CK(launch_c_backward<double>(op.cf, op.wf, op.xf, y, ld, nrhs, st));
         return SLR_OK;
     }
     DevOperator<float>& op = h->op32;
     CK(launch_convert<double, float>(s, nrhs, g, ld, op.gp, s, st));
+    DepScope dep(st);
     CK(launch_c_forward<float>(op.cf, op.gp, s, op.wf, nrhs, st));
     if (lowrank) CK(launch_lowrank<float>(op, s, h->k, op.wf, nrhs, st));
     CK(launch_c_backward<float>(op.cf, op.wf, op.xf, op.gp, s, nrhs, st));

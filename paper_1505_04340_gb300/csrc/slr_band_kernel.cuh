@@ -190,7 +190,11 @@ k_band_wide(const BandBlock* __restrict__ blocks, const T* __restrict__ fac, con
     const int g = (G > 1) ? (int)cg::this_cluster().block_rank() : 0;
     const BandBlock& b = blocks[sub];
     const int W = b.w, c = b.c, m = b.m, WP = (W + 3) & ~3;
-    if (m == 0) return;                         // uniform across the cluster
+    dep_go();
+    if (m == 0) {                               // uniform across the cluster
+        dep_wait();
+        return;
+    }
     const int SU = b.SU, SL = b.SL, row0 = b.row0, nrb = b.nrb[g];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
@@ -382,6 +386,7 @@ k_band_wide(const BandBlock* __restrict__ blocks, const T* __restrict__ fac, con
 
     if (lane == 0)
         while (issued < nbuf && iplane >= 0) issue_next();
+    dep_wait();                                          // (the copies so far are of the factor)
     // every CTA of the cluster has armed its barriers before any st.async reaches it
     cluster_barrier<G>();
 
@@ -606,13 +611,18 @@ cudaError_t band_launch(const DevOperator<T>& op, int32_t p, int32_t wmax, const
     cfg.blockDim = dim3(NT);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = G;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
+    int na = G > 1 ? 1 : 0;
+    if (dep_active()) {
+        attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[na++].val.programmaticStreamSerializationAllowed = 1;
+    }
     cfg.attrs = attr;
-    cfg.numAttrs = G > 1 ? 1 : 0;
+    cfg.numAttrs = na;
     e = cudaLaunchKernelEx(&cfg, kern, op.band, op.bfac, in, ldi, out, ldo, base, ldb, op.err, nr, (int)nbuf, (int)cq, op.bfac_len * (int64_t)sizeof(T) > kL2Keep ? 1 : 0);
     count_launches(1);
     return e;

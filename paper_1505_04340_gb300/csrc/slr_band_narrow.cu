@@ -73,7 +73,11 @@ k_band_narrow(const BandBlock* __restrict__ blocks, const T* __restrict__ fac, c
     constexpr int PB = kNw * NR * 64;                  // partial sums of a block
     extern __shared__ __align__(128) unsigned char smem[];
     const int W = blocks[blockIdx.x].w, c = blocks[blockIdx.x].c, m = blocks[blockIdx.x].m;
-    if (m == 0) return;
+    dep_go();
+    if (m == 0) {
+        dep_wait();
+        return;
+    }
     const int SU = blocks[blockIdx.x].SU, SL = blocks[blockIdx.x].SL;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     uint64_t* full = reinterpret_cast<uint64_t*>(smem);                      // [kNSlots]
@@ -127,6 +131,7 @@ k_band_narrow(const BandBlock* __restrict__ blocks, const T* __restrict__ fac, c
         return;
     }
     // ------------------------------------------------------------------ products
+    dep_wait();                                          // (the copy warp reads the factor only)
     const bool two = W > 32;
     T* vw = part + 2 * PB + warp * kNc * NR;             // [kNc][NR] this warp's entries of the input vector
     // the lane's pairs: column (past W: none), right-hand side; only the last plane has rows past m
@@ -334,9 +339,9 @@ cudaError_t narrow_launch(const DevOperator<T>& op, int32_t p, int32_t wmax, con
     const int32_t nslot =
         std::max<int32_t>(2, std::min<int32_t>(kNSlots, (int32_t)((budget - std::min(budget, fixed)) / sb)));
     if (fixed + (size_t)nslot * sb > kCap) return cudaErrorInvalidValue;
-    kern<<<p, 32 * (kNw + 1), fixed + (size_t)nslot * sb, st>>>(op.band, op.bfac, in, ldi, out, ldo, base, ldb, op.err,
-                                                                 nslot, slot,
-                                                                 op.bfac_len * (int64_t)sizeof(T) > kL2Keep ? 1 : 0);
+    const cudaError_t e = launch_dep(kern, p, 32 * (kNw + 1), fixed + (size_t)nslot * sb, st, op.band, op.bfac, in, ldi, out,
+                                     ldo, base, ldb, op.err, nslot, slot, op.bfac_len * (int64_t)sizeof(T) > kL2Keep ? 1 : 0);
+    if (e != cudaSuccess) return e;
     count_launches(1);
     return cudaGetLastError();
 }

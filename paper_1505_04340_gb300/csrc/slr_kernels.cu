@@ -29,6 +29,23 @@ void count_launches(int64_t n) {
     g_kernel_launches.fetch_add(n, std::memory_order_relaxed);
     t_kernel_launches += n;
 }
+namespace {
+thread_local bool t_dep = false;
+}
+bool dep_active() { return t_dep; }
+DepScope::DepScope(cudaStream_t st, bool on) : before_(t_dep) {
+    if (on && st) {                          // (the default stream is never captured)
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) {
+            cudaGetLastError();
+            on = false;
+        }
+        on = on && cs == cudaStreamCaptureStatusNone;
+    }
+    t_dep = on;
+}
+DepScope::~DepScope() { t_dep = before_; }
+
 int64_t thread_launches() { return t_kernel_launches; }
 
 namespace {
@@ -94,6 +111,8 @@ template <typename T>
 __global__ void k_spmv_cols(int32_t rows, int32_t nrhs, const int32_t* __restrict__ rp,
                             const int32_t* __restrict__ ci, const T* __restrict__ v, const T* x, int64_t ldx,
                             const T* g, int64_t ldg, T* y, int64_t ldy) {
+    dep_go();
+    dep_wait();
     const int32_t ngr = (nrhs + kSpCols - 1) / kSpCols;
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= (int64_t)rows * ngr) return;
@@ -1034,6 +1053,7 @@ __device__ void cfwd_small_cta(const CView<T>& cf, int J, T* ts, const T* g, int
     const int64_t nr = cf.r_off[J + 1] - cf.r_off[J], rtot = nJ + nr;
     const T *D, *Pn;
     const bool staged = stage_block_fwd<T, NT>(cf, J, stg, cap, gt, D, Pn);   // lands while t_J is gathered
+    dep_wait();                                                             // (the factor is nobody's output)
     if constexpr (TILED) {
         if (staged) {
             cfwd_small_tiled<T, NT, GROUPS>(cf, J, ts, g, ldg, xf, nrhs, D, Pn);
@@ -1287,6 +1307,7 @@ __device__ void cbwd_small_cta(const CView<T>& cf, int J, T* vs, T* red, const T
     const int32_t* R = cf.rows + cf.r_off[J];
     const T *D, *Pn;
     const bool staged = stage_block<T, NT>(cf, J, stg, cap, gt, D, Pn);   // lands while the vector is staged
+    dep_wait();                                                         // (the factor is nobody's output)
     if constexpr (TILED) {
         // right-hand sides per pass: the vector (rows x RP) and the sums (NT x RP) fit the buffer
         const int rpm = min(tile_rp<T>(), (int)(tile_vs<T>() / max(rtot, (int64_t)NT)) & ~7);
@@ -1372,6 +1393,8 @@ template <typename T, int NW>
 __global__ void __launch_bounds__(NW * 32, NW == 8 ? 4 : 1)
 k_cfwd_level(const CView<T> cf, int32_t t0, int32_t p0, int32_t np, const T* g, int64_t ldg, T* xf, int32_t nrhs,
              int32_t tstride, int32_t rbmax) {
+    dep_go();
+    dep_wait();
     extern __shared__ __align__(16) unsigned char csm[];
     __shared__ T red[NW][33];
     const int q = blockIdx.x;
@@ -1389,6 +1412,8 @@ k_cfwd_level(const CView<T> cf, int32_t t0, int32_t p0, int32_t np, const T* g, 
 template <typename T, int NW, int RP, int R>
 __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 1)
 k_cfwd_level_blk(const CView<T> cf, int32_t t0, int32_t p0, int32_t np, T* xf, int32_t nrhs, int32_t tstride) {
+    dep_go();
+    dep_wait();
     extern __shared__ __align__(16) unsigned char csm[];
     const int q = blockIdx.x, j0 = blockIdx.y * RP;
     const bool pan = q < np;
@@ -1403,7 +1428,9 @@ k_cfwd_level_blk(const CView<T> cf, int32_t t0, int32_t p0, int32_t np, T* xf, i
 // transposes them in shared memory and writes each factor-order row's right-hand sides together.
 template <typename T>
 __global__ void __launch_bounds__(256)
-k_cperm_g(int32_t s, int32_t nrhs, const int32_t* __restrict__ ciperm, const T* __restrict__ g, int64_t ldg, T* gf) {
+k_cperm_g(int32_t s, int32_t nrhs, const int32_t* __restrict__ ciperm, const T* g, int64_t ldg, T* gf) {
+    dep_go();
+    dep_wait();
     __shared__ T tile[32][33];
     const int i0 = blockIdx.x * 32, j0 = blockIdx.y * 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
 #pragma unroll
@@ -1424,7 +1451,9 @@ k_cperm_g(int32_t s, int32_t nrhs, const int32_t* __restrict__ ciperm, const T* 
 // row of xf is read as whole lines here, and y written along i.
 template <typename T>
 __global__ void __launch_bounds__(256)
-k_cperm_y(int32_t s, int32_t nrhs, const int32_t* __restrict__ ciperm, const T* __restrict__ xf, T* y, int64_t ldy) {
+k_cperm_y(int32_t s, int32_t nrhs, const int32_t* __restrict__ ciperm, const T* xf, T* y, int64_t ldy) {
+    dep_go();
+    dep_wait();
     __shared__ T tile[32][33];
     const int i0 = blockIdx.x * 32, j0 = blockIdx.y * 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
 #pragma unroll
@@ -1447,6 +1476,8 @@ k_cperm_y(int32_t s, int32_t nrhs, const int32_t* __restrict__ ciperm, const T* 
 template <typename T>
 __global__ void __launch_bounds__(256)
 k_cfwd_gather(const CView<T> cf, int32_t s0, const T* g, int64_t ldg, int32_t nrhs) {
+    dep_go();
+    dep_wait();
     const int32_t J = cf.lev_sn[s0 + blockIdx.x];
     const int32_t a0 = cf.c0[J], nJ = cf.c0[J + 1] - a0;
     const int64_t e = (int64_t)blockIdx.y * 256 + threadIdx.x;
@@ -1463,6 +1494,8 @@ k_cfwd_gather(const CView<T> cf, int32_t s0, const T* g, int64_t ldg, int32_t nr
 template <typename T, int NW>
 __global__ void __launch_bounds__(NW * 32, NW == 8 ? 4 : 1)
 k_cbwd_level(const CView<T> cf, int32_t t0, const T* yf, T* xf, T* y_dd, int64_t ldy, int32_t nrhs) {
+    dep_go();
+    dep_wait();
     extern __shared__ __align__(16) unsigned char csm[];
     __shared__ T red[NW][33];
     __shared__ T us[8 * 32];
@@ -1477,6 +1510,8 @@ k_cbwd_level(const CView<T> cf, int32_t t0, const T* yf, T* xf, T* y_dd, int64_t
 template <typename T, int NW, int RP>
 __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 1)
 k_cbwd_level_blk(const CView<T> cf, int32_t t0, const T* yf, T* xf, T* y_dd, int64_t ldy, int32_t nrhs, int ystage) {
+    dep_go();
+    dep_wait();
     extern __shared__ __align__(16) unsigned char csm[];
     T* us = reinterpret_cast<T*>(csm);
     T* xs = us + RP * 32;
@@ -1497,6 +1532,7 @@ template <typename T, int RB, bool TILED>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 2)
 k_cfwd_small(const CView<T> cf, int32_t s0, const T* g, int64_t ldg, T* xf, int32_t nrhs, int32_t cap,
              int32_t tsz) {
+    dep_go();
     extern __shared__ __align__(16) unsigned char csm[];
     T* ts = reinterpret_cast<T*>(csm);
     cfwd_small_cta<T, kThreads, 1, RB, TILED>(cf, cf.lev_sn[s0 + blockIdx.x], ts, g, ldg, xf, nrhs, ts + tsz, cap);
@@ -1509,6 +1545,7 @@ template <typename T, int RB, bool TILED>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 2)
 k_cbwd_small(const CView<T> cf, int32_t s0, const T* yf, T* xf, T* y_dd, int64_t ldy, int32_t nrhs, int32_t cap,
              int32_t vsz) {
+    dep_go();
     extern __shared__ __align__(16) unsigned char csm[];
     T* vs = reinterpret_cast<T*>(csm);
     T* red = vs + RB * (kSmallN + kSmallR);
@@ -1523,7 +1560,7 @@ cudaError_t cfwd_small_launch(const CView<T>& v, int s0, int ns, int32_t cap, co
     const size_t sm = ((size_t)tsz + cap) * sizeof(T);
     auto kern = k_cfwd_small<T, RB, TILED>;
     if (sm > 48 * 1024 && !raise_smem_once((const void*)kern)) return cudaErrorInvalidValue;
-    kern<<<ns, kThreads, sm, st>>>(v, s0, g, ldg, xf, nrhs, cap, tsz);
+    launch_dep(kern, ns, kThreads, sm, st, v, s0, g, ldg, xf, nrhs, cap, tsz);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -1534,7 +1571,7 @@ cudaError_t cbwd_small_launch(const CView<T>& v, int s0, int ns, int32_t cap, co
     const size_t sm = ((size_t)vsz + cap) * sizeof(T);
     auto kern = k_cbwd_small<T, RB, TILED>;
     if (sm > 48 * 1024 && !raise_smem_once((const void*)kern)) return cudaErrorInvalidValue;
-    kern<<<ns, kThreads, sm, st>>>(v, s0, yf, xf, y_dd, ldy, nrhs, cap, vsz);
+    launch_dep(kern, ns, kThreads, sm, st, v, s0, yf, xf, y_dd, ldy, nrhs, cap, vsz);
     count_launches(1);
     return cudaGetLastError();
 }
@@ -1548,6 +1585,8 @@ constexpr int kTopT = 256;   // threads of the zone kernels (8 warps)
 template <typename T>
 __global__ void __launch_bounds__(kThreads)
 k_ctop_gather(const CView<T> cf, const T* g, int64_t ldg, int32_t nrhs) {
+    dep_go();
+    dep_wait();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (int64_t)cf.nT * nrhs) return;
     const int32_t la = (int32_t)(i / nrhs), j = (int32_t)(i - (int64_t)la * nrhs);
@@ -1590,6 +1629,8 @@ constexpr int kTopR = sizeof(T) == 4 ? 8 : 4;
 template <typename T, int RB>
 __global__ void __launch_bounds__(kTopT)
 k_ctop_fwd(const CView<T> cf, T* xf, int32_t nrhs) {
+    dep_go();
+    dep_wait();
     __shared__ T ts[RB][kTopCW];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int4 tk = cf.tf_tasks[blockIdx.x];
@@ -1658,6 +1699,8 @@ k_ctop_fwd(const CView<T> cf, T* xf, int32_t nrhs) {
 template <typename T, int RB>
 __global__ void __launch_bounds__(kTopT)
 k_ctop_bwd(const CView<T> cf, const T* yf, T* xf, T* y_dd, int64_t ldy, int32_t nrhs) {
+    dep_go();
+    dep_wait();
     constexpr int NW = kTopT / 32, DEPTH = sizeof(T) == 4 ? 16 : 8;
     __shared__ __align__(16) T xs[kTopRCH * RB];
     __shared__ T red[NW][RB][33];
@@ -1853,7 +1896,9 @@ __host__ __device__ inline int lr_blocks(int32_t s) {
 // turns into the CTA's partial sums.  The order of every sum depends on s only.
 template <typename T>
 __global__ void __launch_bounds__(256)
-k_lr_vt(int32_t s, int32_t k, int32_t nrhs, const T* __restrict__ U, const T* __restrict__ w, int64_t ldw, T* part) {
+k_lr_vt(int32_t s, int32_t k, int32_t nrhs, const T* __restrict__ U, const T* w, int64_t ldw, T* part) {
+    dep_go();
+    dep_wait();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int R = (s + gridDim.x - 1) / gridDim.x;
     const int r0 = blockIdx.x * R, r1 = min(s, r0 + R);
@@ -1904,7 +1949,9 @@ k_lr_vt(int32_t s, int32_t k, int32_t nrhs, const T* __restrict__ U, const T* __
 constexpr int kLrSeg = 16, kLrFinJ = 16;
 template <typename T>
 __global__ void __launch_bounds__(kLrSeg * kLrFinJ)
-k_lr_vt_fin(int32_t k, int32_t nrhs, int32_t G, const T* __restrict__ part, const T* __restrict__ dvec, T* vk) {
+k_lr_vt_fin(int32_t k, int32_t nrhs, int32_t G, const T* part, const T* __restrict__ dvec, T* vk) {
+    dep_go();
+    dep_wait();
     __shared__ T seg[kLrSeg][kLrFinJ];
     const int kk = blockIdx.x, jl = threadIdx.x % kLrFinJ, q = threadIdx.x / kLrFinJ;
     const int j = blockIdx.y * kLrFinJ + jl;
@@ -1933,8 +1980,10 @@ k_lr_vt_fin(int32_t k, int32_t nrhs, int32_t G, const T* __restrict__ part, cons
 // thread = row i, JG right-hand sides (a block's columns j0 .. j0 + JG - 1 of nrhs)
 template <typename T, int JG>
 __global__ void __launch_bounds__(256)
-k_lr_update(int32_t s, int32_t k, int32_t nrhs, const T* __restrict__ U, const T* __restrict__ vk, T cinv, T* w,
+k_lr_update(int32_t s, int32_t k, int32_t nrhs, const T* __restrict__ U, const T* vk, T cinv, T* w,
             int64_t ldw) {
+    dep_go();
+    dep_wait();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= s) return;
     const int j0 = blockIdx.y * JG;
@@ -1952,13 +2001,13 @@ k_lr_update(int32_t s, int32_t k, int32_t nrhs, const T* __restrict__ U, const T
         for (int e = 0; e < 8; ++e)
 #pragma unroll
             for (int q = 0; q < JG; ++q)
-                if (q < jn) acc[q] = fma(u[e], __ldg(&vk[kk + e + (int64_t)(j0 + q) * k]), acc[q]);
+                if (q < jn) acc[q] = fma(u[e], vk[kk + e + (int64_t)(j0 + q) * k], acc[q]);
     }
     for (; kk < k; ++kk) {
         const T u = U[i + (int64_t)kk * s];
 #pragma unroll
         for (int q = 0; q < JG; ++q)
-            if (q < jn) acc[q] = fma(u, __ldg(&vk[kk + (int64_t)(j0 + q) * k]), acc[q]);
+            if (q < jn) acc[q] = fma(u, vk[kk + (int64_t)(j0 + q) * k], acc[q]);
     }
 #pragma unroll
     for (int q = 0; q < JG; ++q)
@@ -1972,7 +2021,9 @@ k_lr_update(int32_t s, int32_t k, int32_t nrhs, const T* __restrict__ U, const T
 constexpr int kConvN = 4 * kThreads;
 template <typename TS, typename TD>
 __global__ void __launch_bounds__(kThreads)
-k_convert(int64_t rows, int32_t cols, const TS* __restrict__ src, int64_t lds, TD* __restrict__ dst, int64_t ldd) {
+k_convert(int64_t rows, int32_t cols, const TS* src, int64_t lds, TD* dst, int64_t ldd) {
+    dep_go();
+    dep_wait();
     const int64_t i0 = (int64_t)blockIdx.x * kConvN + threadIdx.x;
     for (int64_t j = blockIdx.y; j < cols; j += gridDim.y) {
         const TS* s = src + j * lds;
@@ -2201,7 +2252,7 @@ cudaError_t spmv_cols(int32_t rows, int32_t nrhs, const int32_t* rp, const int32
                       int64_t ldx, const T* g, int64_t ldg, T* y, int64_t ldy, cudaStream_t st) {
     if (rows == 0 || nrhs == 0) return cudaSuccess;
     const int64_t threads = (int64_t)rows * ((nrhs + kSpCols - 1) / kSpCols);
-    k_spmv_cols<T><<<blocks_for(threads), kThreads, 0, st>>>(rows, nrhs, rp, ci, v, x, ldx, g, ldg, y, ldy);
+    launch_dep(k_spmv_cols<T>, blocks_for(threads), kThreads, 0, st, rows, nrhs, rp, ci, v, x, ldx, g, ldg, y, ldy);
     counted();
     return cudaGetLastError();
 }
@@ -2352,7 +2403,7 @@ cudaError_t launch_c_forward(const DevCFactor<T>& cf, const T* g_dd, int64_t ldg
     v.wr = nrhs;     // wbuf and tws: a call's right-hand sides contiguous per row (one line per gathered row)
     if (nrhs >= 8 && cf.gfs && cf.s > 0) {
         // blocks: g in factor order, a row per position, so every gather of g reads whole lines
-        k_cperm_g<T><<<dim3((cf.s + 31) / 32, (nrhs + 31) / 32), 256, 0, st>>>(cf.s, nrhs, cf.ciperm, g_dd, ldg,
+        launch_dep(k_cperm_g<T>, dim3((cf.s + 31) / 32, (nrhs + 31) / 32), 256, 0, st, cf.s, nrhs, cf.ciperm, g_dd, ldg,
                                                                                cf.gfs);
         counted();
         v.gf = cf.gfs;
@@ -2395,7 +2446,7 @@ cudaError_t launch_c_forward(const DevCFactor<T>& cf, const T* g_dd, int64_t ldg
             vl.tws = cf.tws;                  // the gather writes it, the level's tasks read it
             const int s0 = cf.lev_sn_ptr[l], ns = cf.lev_sn_ptr[l + 1] - s0;
             const unsigned chunks = (unsigned)(((int64_t)cf.lev_maxn[l] * nrhs + 255) / 256);
-            k_cfwd_gather<T><<<dim3(ns, chunks), 256, 0, st>>>(vl, s0, g_dd, ldg, nrhs);
+            launch_dep(k_cfwd_gather<T>, dim3(ns, chunks), 256, 0, st, vl, s0, g_dd, ldg, nrhs);
             counted();
         }
         const bool wide = nt + np <= cf.nsm;
@@ -2408,7 +2459,7 @@ cudaError_t launch_c_forward(const DevCFactor<T>& cf, const T* g_dd, int64_t ldg
             auto blk = [&](auto kern, int rp, int nw) -> bool {
                 const size_t sm = ((size_t)ts_n * (rp + 4) + (size_t)nw * rp * 32) * sizeof(T);
                 if (sm > kLevSmem || (sm > 48 * 1024 && !raise_smem_once((const void*)kern))) return false;
-                kern<<<dim3(nt + np, (nrhs + rp - 1) / rp), nw * 32, sm, st>>>(vl, t0, p0, np, xf, nrhs, ts_n);
+                launch_dep(kern, dim3(nt + np, (nrhs + rp - 1) / rp), nw * 32, sm, st, vl, t0, p0, np, xf, nrhs, ts_n);
                 counted();
                 return true;
             };
@@ -2434,17 +2485,17 @@ cudaError_t launch_c_forward(const DevCFactor<T>& cf, const T* g_dd, int64_t ldg
         const size_t smem = need(rbmax);
         if (smem > 48 * 1024 && !raise_smem_once(kern)) return cudaErrorInvalidValue;
         if (!wide)
-            k_cfwd_level<T, 8><<<nt + np, 256, smem, st>>>(vl, t0, p0, np, g_dd, ldg, xf, nrhs, cf.max_n, rbmax);
+            launch_dep(k_cfwd_level<T, 8>, nt + np, 256, smem, st, vl, t0, p0, np, g_dd, ldg, xf, nrhs, cf.max_n, rbmax);
         else
-            k_cfwd_level<T, 32><<<nt + np, 1024, smem, st>>>(vl, t0, p0, np, g_dd, ldg, xf, nrhs, cf.max_n, rbmax);
+            launch_dep(k_cfwd_level<T, 32>, nt + np, 1024, smem, st, vl, t0, p0, np, g_dd, ldg, xf, nrhs, cf.max_n, rbmax);
         counted();
     }
     if (cf.nT > 0) {
-        k_ctop_gather<T><<<blocks_for((int64_t)cf.nT * nrhs), kThreads, 0, st>>>(v, g_dd, ldg, nrhs);
-        if (nrhs == 1) k_ctop_fwd<T, 1><<<cf.n_tf_tasks, kTopT, 0, st>>>(v, xf, nrhs);
-        else if (nrhs == 2) k_ctop_fwd<T, 2><<<cf.n_tf_tasks, kTopT, 0, st>>>(v, xf, nrhs);
-        else if (nrhs <= 4) k_ctop_fwd<T, 4><<<cf.n_tf_tasks, kTopT, 0, st>>>(v, xf, nrhs);
-        else k_ctop_fwd<T, kTopR<T>><<<cf.n_tf_tasks, kTopT, 0, st>>>(v, xf, nrhs);
+        launch_dep(k_ctop_gather<T>, blocks_for((int64_t)cf.nT * nrhs), kThreads, 0, st, v, g_dd, ldg, nrhs);
+        if (nrhs == 1) launch_dep(k_ctop_fwd<T, 1>, cf.n_tf_tasks, kTopT, 0, st, v, xf, nrhs);
+        else if (nrhs == 2) launch_dep(k_ctop_fwd<T, 2>, cf.n_tf_tasks, kTopT, 0, st, v, xf, nrhs);
+        else if (nrhs <= 4) launch_dep(k_ctop_fwd<T, 4>, cf.n_tf_tasks, kTopT, 0, st, v, xf, nrhs);
+        else launch_dep(k_ctop_fwd<T, kTopR<T>>, cf.n_tf_tasks, kTopT, 0, st, v, xf, nrhs);
         counted(2);
     }
     return cudaGetLastError();
@@ -2457,10 +2508,10 @@ cudaError_t c_backward_steps(const DevCFactor<T>& cf, const T* yf, T* xf, T* y_d
     CView<T> v = make_view(cf, cf.nsteps_bwd);
     v.xr = nrhs;     // the solution x (scratch): a call's right-hand sides contiguous per row
     if (cf.nT > 0) {
-        if (nrhs == 1) k_ctop_bwd<T, 1><<<cf.n_tb_tasks, kTopT, 0, st>>>(v, yf, xf, y_dd, ldy, nrhs);
-        else if (nrhs == 2) k_ctop_bwd<T, 2><<<cf.n_tb_tasks, kTopT, 0, st>>>(v, yf, xf, y_dd, ldy, nrhs);
-        else if (nrhs <= 4) k_ctop_bwd<T, 4><<<cf.n_tb_tasks, kTopT, 0, st>>>(v, yf, xf, y_dd, ldy, nrhs);
-        else k_ctop_bwd<T, kTopR<T>><<<cf.n_tb_tasks, kTopT, 0, st>>>(v, yf, xf, y_dd, ldy, nrhs);
+        if (nrhs == 1) launch_dep(k_ctop_bwd<T, 1>, cf.n_tb_tasks, kTopT, 0, st, v, yf, xf, y_dd, ldy, nrhs);
+        else if (nrhs == 2) launch_dep(k_ctop_bwd<T, 2>, cf.n_tb_tasks, kTopT, 0, st, v, yf, xf, y_dd, ldy, nrhs);
+        else if (nrhs <= 4) launch_dep(k_ctop_bwd<T, 4>, cf.n_tb_tasks, kTopT, 0, st, v, yf, xf, y_dd, ldy, nrhs);
+        else launch_dep(k_ctop_bwd<T, kTopR<T>>, cf.n_tb_tasks, kTopT, 0, st, v, yf, xf, y_dd, ldy, nrhs);
         counted();
     }
     if (cf.nsteps_bwd == 0) return cudaGetLastError();
@@ -2496,7 +2547,7 @@ cudaError_t c_backward_steps(const DevCFactor<T>& cf, const T* yf, T* xf, T* y_d
                 const bool ystage = full <= kLevSmem;
                 const size_t sm = ystage ? full : base;
                 if (sm > kLevSmem || (sm > 48 * 1024 && !raise_smem_once((const void*)kern))) return false;
-                kern<<<dim3(nt, (nrhs + rp - 1) / rp), nw * 32, sm, st>>>(v, t0, yf, xf, y_dd, ldy, nrhs, ystage ? 1 : 0);
+                launch_dep(kern, dim3(nt, (nrhs + rp - 1) / rp), nw * 32, sm, st, v, t0, yf, xf, y_dd, ldy, nrhs, ystage ? 1 : 0);
                 counted();
                 return true;
             };
@@ -2511,11 +2562,11 @@ cudaError_t c_backward_steps(const DevCFactor<T>& cf, const T* yf, T* xf, T* y_d
         // blocks of four or more: the panel part's partial sums, NW x 8 x 32
         if (nt > cf.nsm) {
             const size_t sm = nrhs >= 4 ? (size_t)8 * 8 * 32 * sizeof(T) : 0;
-            k_cbwd_level<T, 8><<<nt, 256, sm, st>>>(v, t0, yf, xf, y_dd, ldy, nrhs);
+            launch_dep(k_cbwd_level<T, 8>, nt, 256, sm, st, v, t0, yf, xf, y_dd, ldy, nrhs);
         } else {
             const size_t sm = nrhs >= 4 ? (size_t)32 * 8 * 32 * sizeof(T) : 0;
             if (sm > 48 * 1024 && !raise_smem_once((const void*)k_cbwd_level<T, 32>)) return cudaErrorInvalidValue;
-            k_cbwd_level<T, 32><<<nt, 1024, sm, st>>>(v, t0, yf, xf, y_dd, ldy, nrhs);
+            launch_dep(k_cbwd_level<T, 32>, nt, 1024, sm, st, v, t0, yf, xf, y_dd, ldy, nrhs);
         }
         counted();
     }
@@ -2531,7 +2582,7 @@ cudaError_t launch_c_backward(const DevCFactor<T>& cf, const T* yf, T* xf, T* y_
     const bool after = nrhs >= 8 && (int64_t)cf.s * nrhs >= 1 << 20 && y_dd && cf.ciperm;
     const cudaError_t e = c_backward_steps<T>(cf, yf, xf, after ? nullptr : y_dd, ldy, nrhs, st);
     if (e != cudaSuccess || !after) return e;
-    k_cperm_y<T><<<dim3((cf.s + 31) / 32, (nrhs + 31) / 32), 256, 0, st>>>(cf.s, nrhs, cf.ciperm, xf, y_dd, ldy);
+    launch_dep(k_cperm_y<T>, dim3((cf.s + 31) / 32, (nrhs + 31) / 32), 256, 0, st, cf.s, nrhs, cf.ciperm, xf, y_dd, ldy);
     counted();
     return cudaGetLastError();
 }
@@ -2545,8 +2596,8 @@ cudaError_t launch_lowrank_v(const DevOperator<T>& op, int32_t s, int32_t k, con
                              int32_t nrhs, cudaStream_t st) {
     if (s == 0 || k == 0) return cudaSuccess;
     const int G = lr_blocks(s);
-    k_lr_vt<T><<<G, 256, 0, st>>>(s, k, nrhs, Ub, w, ldw, op.part);
-    k_lr_vt_fin<T><<<dim3(k, (nrhs + kLrFinJ - 1) / kLrFinJ), kLrSeg * kLrFinJ, 0, st>>>(k, nrhs, G, op.part, op.dvec,
+    launch_dep(k_lr_vt<T>, G, 256, 0, st, s, k, nrhs, Ub, w, ldw, op.part);
+    launch_dep(k_lr_vt_fin<T>, dim3(k, (nrhs + kLrFinJ - 1) / kLrFinJ), kLrSeg * kLrFinJ, 0, st, k, nrhs, G, op.part, op.dvec,
                                                                                         op.vk);
     counted(2);
     return cudaGetLastError();
@@ -2559,11 +2610,11 @@ cudaError_t launch_lowrank_update(const DevOperator<T>& op, int32_t s, int32_t k
     const dim3 grid((unsigned)((s + 255) / 256));
     // every column sees the same multiply-adds in the same order whatever JG is
     if (nrhs == 1) {
-        k_lr_update<T, 1><<<grid, 256, 0, st>>>(s, k, nrhs, Ub, op.vk, op.cinv, w, ldw);
+        launch_dep(k_lr_update<T, 1>, grid, 256, 0, st, s, k, nrhs, Ub, op.vk, op.cinv, w, ldw);
     } else if (nrhs <= 8) {
-        k_lr_update<T, 8><<<grid, 256, 0, st>>>(s, k, nrhs, Ub, op.vk, op.cinv, w, ldw);
+        launch_dep(k_lr_update<T, 8>, grid, 256, 0, st, s, k, nrhs, Ub, op.vk, op.cinv, w, ldw);
     } else {
-        k_lr_update<T, 32><<<dim3(grid.x, (nrhs + 31) / 32), 256, 0, st>>>(s, k, nrhs, Ub, op.vk, op.cinv, w, ldw);
+        launch_dep(k_lr_update<T, 32>, dim3(grid.x, (nrhs + 31) / 32), 256, 0, st, s, k, nrhs, Ub, op.vk, op.cinv, w, ldw);
     }
     counted();
     return cudaGetLastError();
@@ -2587,7 +2638,7 @@ template <typename TS, typename TD>
 cudaError_t launch_convert(int64_t rows, int32_t cols, const TS* src, int64_t lds, TD* dst, int64_t ldd,
                            cudaStream_t st) {
     if (rows * cols == 0) return cudaSuccess;
-    k_convert<TS, TD><<<dim3(blocks_for(rows, kConvN), std::min(cols, 65535)), kThreads, 0, st>>>(rows, cols, src, lds,
+    launch_dep(k_convert<TS, TD>, dim3(blocks_for(rows, kConvN), std::min(cols, 65535)), kThreads, 0, st, rows, cols, src, lds,
                                                                                                dst, ldd);
     counted();
     return cudaGetLastError();
