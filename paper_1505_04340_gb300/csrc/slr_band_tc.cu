@@ -193,6 +193,8 @@ __global__ void __launch_bounds__(kBtThreads, NP <= 32 ? 2 : 1)
 k_band_tc(const BandTcBlock* __restrict__ blocks, const unsigned char* __restrict__ fac, const float* in,
           int64_t ldi, float* out, int64_t ldo, const float* base, int64_t ldb, int32_t nrhs, int32_t nslot,
           int32_t stiles, int32_t* err) {
+    dep_go();
+    dep_wait();
     using Tp = BtType<AB>;
     using Te = typename Tp::Te;
     constexpr int E = Tp::E, KS = Tp::KS;
@@ -505,10 +507,10 @@ cudaError_t bt_launch(const DevOperator<float>& op, int32_t p, const float* in, 
     const size_t smem = (size_t)nslot * stiles * kSub + fixed;
     cudaError_t e = cudaFuncSetAttribute(k_band_tc<AB, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     if (e != cudaSuccess) return e;
-    k_band_tc<AB, NP><<<p, kBtThreads, smem, st>>>(op.band_tc, op.band_tc_fac, in, ldi, out, ldo, base, ldb, nrhs,
-                                                  nslot, stiles, op.err);
+    e = launch_dep(k_band_tc<AB, NP>, p, kBtThreads, smem, st, op.band_tc, op.band_tc_fac, in, ldi, out, ldo, base, ldb,
+                   nrhs, nslot, stiles, op.err);
     count_launches(1);
-    return cudaGetLastError();
+    return e;
 }
 
 template <int AB>

@@ -62,7 +62,9 @@ __host__ __device__ inline int tc_blocks(int32_t s) {
 template <int AB, int UK, int WK>
 __global__ void __launch_bounds__(kTcThreads, 1)
 k_lr_vt_tc(int32_t s, int32_t k, int32_t nrhs, int32_t np, const typename TcType<AB>::U* __restrict__ Ucm,
-           const float* __restrict__ w, float* part, int32_t* err) {
+           const float* w, float* part, int32_t* err) {
+    dep_go();
+    dep_wait();
     using Tp = TcType<AB>;
     using Te = typename Tp::U;
     constexpr int E = Tp::E;
@@ -85,9 +87,8 @@ k_lr_vt_tc(int32_t s, int32_t k, int32_t nrhs, int32_t np, const typename TcType
         tc::mbar_init(&bar[2], 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    // rows k .. 127 of A and nrhs .. np-1 of B stay zero in both stages
-    for (int i = t; i < (int)(2 * kA + 2 * kB) / 16; i += kTcThreads)
-        reinterpret_cast<uint4*>(sm)[i] = make_uint4(0, 0, 0, 0);
+    // (rows k .. 127 of A and nrhs .. np-1 of B are never written: they reach only the rows and
+    // columns of the product that nobody reads)
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
@@ -179,7 +180,9 @@ k_lr_vt_tc(int32_t s, int32_t k, int32_t nrhs, int32_t np, const typename TcType
 template <int AB>
 __global__ void __launch_bounds__(kTcThreads, 1)
 k_lr_update_tc(int32_t s, int32_t k, int32_t kp, int32_t nrhs, int32_t np, const typename TcType<AB>::U* __restrict__ Urm,
-               const float* __restrict__ vk, float cinv, float* w, int32_t* err) {
+               const float* vk, float cinv, float* w, int32_t* err) {
+    dep_go();
+    dep_wait();
     using Tp = TcType<AB>;
     using Te = typename Tp::U;
     constexpr int E = Tp::E;
@@ -202,7 +205,35 @@ k_lr_update_tc(int32_t s, int32_t k, int32_t kp, int32_t nrhs, int32_t np, const
     }
     const int64_t i0 = (int64_t)blockIdx.x * M;
     const int rows = (int)((s - i0) < M ? (s - i0) : M);
+    // this thread's row of w, first 32 columns: on its way while U is staged and multiplied
+    const int wrow = 32 * warp + lane;
+    float o[32];
+#pragma unroll
+    for (int j = 0; j < 32; ++j) o[j] = (wrow < rows && j < nrhs) ? w[i0 + wrow + (int64_t)j * s] : 0.0f;
     // rows of U: sixteen loads in flight per thread before any is stored
+    if (AB == 2 && k % 4 == 0) {
+        // whole 16-byte words, which the operand layout keeps whole (one value at a time took two
+        // divisions per value: with no zeroed operands in pass 1, PCG on FV 96^3 with 32 columns 92.3 -> 91.9 ms)
+        const int nv = kp / 4;
+        for (int e0 = t; e0 < M * nv; e0 += 8 * kTcThreads) {
+            float4 v[8];
+            int r[8], q[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int e = e0 + u * kTcThreads;
+                r[u] = e / nv;
+                q[u] = 4 * (e - r[u] * nv);
+                v[u] = (r[u] < rows && q[u] < k)
+                           ? *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(Urm) + (i0 + r[u]) * k + q[u])
+                           : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (r[u] < M)
+                    *reinterpret_cast<float4*>(sA + tc::kmajor_off<E>(r[u], q[u], kp)) =
+                        make_float4(tc::to_tf32(v[u].x), tc::to_tf32(v[u].y), tc::to_tf32(v[u].z), tc::to_tf32(v[u].w));
+        }
+    } else
     for (int e0 = t; e0 < M * kp; e0 += 16 * kTcThreads) {
         float v[16];
 #pragma unroll
@@ -239,14 +270,15 @@ k_lr_update_tc(int32_t s, int32_t k, int32_t kp, int32_t nrhs, int32_t np, const
         if (t == 0) atomicExch(err, 3);
     } else {
         tc::fence_after_sync();
-        const int r = 32 * warp + lane;
+        const int r = wrow;
         for (int c = 0; c < np; c += 32) {
             float v[32];
             tc::tmem_ld32(tmem + ((uint32_t)(32 * warp) << 16) + (uint32_t)c, v);
             if (r < rows) {
-                float o[32];
+                if (c > 0) {
 #pragma unroll
-                for (int j = 0; j < 32; ++j) o[j] = c + j < nrhs ? w[i0 + r + (int64_t)(c + j) * s] : 0.0f;
+                    for (int j = 0; j < 32; ++j) o[j] = c + j < nrhs ? w[i0 + r + (int64_t)(c + j) * s] : 0.0f;
+                }
 #pragma unroll
                 for (int j = 0; j < 32; ++j)
                     if (c + j < nrhs) w[i0 + r + (int64_t)(c + j) * s] = cinv * o[j] + v[j];
@@ -267,8 +299,9 @@ k_lr_update_tc(int32_t s, int32_t k, int32_t kp, int32_t nrhs, int32_t np, const
 // added in order
 constexpr int kFinSeg = 16, kFinJ = 16;
 __global__ void __launch_bounds__(kFinSeg * kFinJ)
-k_lr_fin_tc(int32_t k, int32_t nrhs, int32_t G, const float* __restrict__ part, const float* __restrict__ dvec,
-            float* vk) {
+k_lr_fin_tc(int32_t k, int32_t nrhs, int32_t G, const float* part, const float* __restrict__ dvec, float* vk) {
+    dep_go();
+    dep_wait();
     __shared__ float seg[kFinSeg][kFinJ];
     const int kk = blockIdx.x, j = blockIdx.y * kFinJ + (threadIdx.x % kFinJ), q = threadIdx.x / kFinJ;
     const int len = (G + kFinSeg - 1) / kFinSeg, b0 = q * len, b1 = min(G, b0 + len);
@@ -321,8 +354,11 @@ cudaError_t launch_tc(const DevOperator<float>& op, int32_t s, int32_t k, float*
                       : (np <= 32 ? k_lr_vt_tc<AB, 32, 8> : k_lr_vt_tc<AB, 32, 16>);
     cudaError_t e = cudaFuncSetAttribute(vt, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1);
     if (e != cudaSuccess) return e;
-    vt<<<G, kTcThreads, sm1, st>>>(s, k, nrhs, np, Ucm, w, op.part, op.err);
-    k_lr_fin_tc<<<dim3(k, (nrhs + kFinJ - 1) / kFinJ), kFinSeg * kFinJ, 0, st>>>(k, nrhs, G, op.part, op.dvec, op.vk);
+    e = launch_dep(vt, G, kTcThreads, sm1, st, s, k, nrhs, np, Ucm, w, op.part, op.err);
+    if (e != cudaSuccess) return e;
+    e = launch_dep(k_lr_fin_tc, dim3(k, (nrhs + kFinJ - 1) / kFinJ), kFinSeg * kFinJ, 0, st, k, nrhs, G, op.part, op.dvec,
+                   op.vk);
+    if (e != cudaSuccess) return e;
     const int kp = AB == 2 ? (k + 7) / 8 * 8 : (k + 15) / 16 * 16;
     const size_t sm2 = (size_t)(128 + 64) * kp * E + 64;
     // the limit is process-wide state of the kernel: always the same (largest) value,
@@ -330,11 +366,10 @@ cudaError_t launch_tc(const DevOperator<float>& op, int32_t s, int32_t k, float*
     e = cudaFuncSetAttribute(k_lr_update_tc<AB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)((128 + 64) * 128 * E + 64));
     if (e != cudaSuccess) return e;
-    k_lr_update_tc<AB><<<(s + 127) / 128, kTcThreads, sm2, st>>>(s, k, kp, nrhs, np,
-                                                                 reinterpret_cast<const Te*>(op.U_tc_rm), op.vk,
-                                                                 op.cinv, w, op.err);
+    e = launch_dep(k_lr_update_tc<AB>, (s + 127) / 128, kTcThreads, sm2, st, s, k, kp, nrhs, np,
+                   reinterpret_cast<const Te*>(op.U_tc_rm), op.vk, op.cinv, w, op.err);
     count_launches(3);
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace
