@@ -109,7 +109,7 @@ class ClockSampler:
 
 # the source files of each kernel whose ncu traffic a committed summary records
 KERNEL_SOURCES = {
-    "band": ("slr_band_kernel.cuh", "slr_band_half.cu"),       # k_band_solve2 and its instantiations
+    "band": ("slr_band_kernel.cuh", "slr_band_half.cu"),       # k_band_wide and its instantiations
     "band_tc": ("slr_band_tc.cu", "slr_tc.cuh"),
     "csolve": ("slr_kernels.cu",),
     "lowrank": ("slr_kernels.cu",),
@@ -439,8 +439,8 @@ FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e-3
 # ncu summaries under profiles/ that record a kernel's DRAM traffic per launch, by
 # (kernel, workload, precision)
 TRAFFIC_SUMMARIES = {
-    ("band", "3d64", "fp64"): "k_band_solve2_fp64_3d64.txt",
-    ("band", "3d64", "mixed"): "k_band_solve2_fp32_3d64.txt",
+    ("band", "3d64", "fp64"): "k_band_wide_fp64_3d64.txt",
+    ("band", "3d64", "mixed"): "k_band_wide_fp32_3d64.txt",
     ("band_tc", "3d96aniso", "mixed"): "k_band_tc_tf32_3d96aniso_r32.txt",
     ("csolve", "3d96aniso", "mixed"): "c_solve_fp32_3d96aniso_r32.txt",
 }
@@ -483,7 +483,7 @@ def kernel_roofline(kind, info, prec, nrhs, us, hbm, hbm_src, name):
     if kind == "band":        # one B-solve: forward and backward pass over the band factor
         entries = info["band_entries"]
         vec = 2 * info["n_interior"] * nrhs * wf
-        label = "k_band_solve2 (K1, one B-solve)"
+        label = "k_band_wide (K1, one B-solve)"
     else:                     # one C-solve: L^{-1} then L^{-T} (diagonal blocks, panels, top-zone inverse)
         entries = info["c_diag_entries"] + info["c_panel_entries"] + info["c_top_entries"]
         vec = 4 * info["s"] * nrhs * wf

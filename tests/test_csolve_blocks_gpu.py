@@ -27,3 +27,31 @@ def test_csolve_block_widths_equal_single_columns(precision, nrhs):
     for c in {0, 7, nrhs // 2, nrhs - 1}:
         assert np.array_equal(g.csolve(cu(gg[:, c])).cpu().numpy(), y[:, c]), c
     g.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("nrhs", [1, 8])
+@pytest.mark.parametrize("side", [False, True])
+def test_applies_in_a_row_equal_applies_alone(precision, nrhs, side):
+    """An apply's kernels start before the ones ahead of them have ended: calls back to back, each on
+    an input that a kernel on the same stream has just written and into buffers that the call
+    before still uses, give bit for bit what they give one at a time."""
+    P = slrgen.make_problem("m24", (24, 24, 24), (2, 2, 2), 4)
+    g = SLR(P.rowptr, P.colind, P.val, P.part, P.nparts, k=4, lanczos_steps=6, precision=precision, nrhs_max=nrhs)
+    r = cu(np.random.default_rng(3).standard_normal((nrhs, P.n))).t()
+    r = r[:, 0].contiguous() if nrhs == 1 else r
+    with torch.cuda.stream(torch.cuda.Stream() if side else torch.cuda.default_stream()):
+        torch.cuda.synchronize()
+        row, x = [], r
+        for _ in range(8):
+            x = x + g.apply(x)
+            row.append(x)
+        torch.cuda.synchronize()
+        x = r
+        for y in row:
+            z = g.apply(x)
+            torch.cuda.synchronize()
+            x = x + z
+            torch.cuda.synchronize()
+            assert torch.equal(x, y)
+    g.close()
