@@ -344,7 +344,10 @@ k_band_wide(const BandBlock* __restrict__ blocks, const T* __restrict__ fac, con
     // pass's last t and the backward pass's first t have no exchange of y
     // between them, so a fast peer can send the second before a slow CTA has
     // read the first.  y/x needs one buffer (an exchange of t always lies between
-    // two of its phases).  After a wait that expired the barrier
+    // two of its phases).  A slice without rows (planes of fewer than G row blocks)
+    // sends nothing that could hold its peers back: with their next bytes in a phase
+    // it has yet to arm, the phase's count never comes to zero.  So it takes no part: its peers
+    // send it nothing and it waits for nothing.  After a wait that expired the barrier
     // is left un-armed (thread 0 never arrives twice in one phase).
     auto wait_vec = [&](uint64_t* bar, uint32_t par) {
         long long it = 0;
@@ -362,18 +365,24 @@ k_band_wide(const BandBlock* __restrict__ blocks, const T* __restrict__ fac, con
         }
         __syncwarp();
     };
-    // entry (r, j) of a phase's vector vec into every CTA.
-    // An aborted CTA sends nothing more: its peers' waits for its rows then
-    // expire and they abort in turn, so at most a phase or two of bytes reach a
-    // barrier this CTA no longer arms.
-    auto send = [&](T* vec, uint64_t* bar, int j, int r, T v) {
+    unsigned peers = 0;                                   // the other CTAs that own rows
+    if constexpr (G > 1) {
+#pragma unroll
+        for (int pr = 0; pr < G; ++pr)
+            if (pr != g && b.nrb[pr] > 0) peers |= 1u << pr;
+    }
+    // The peers that a phase's rows go to.  An aborted CTA sends nothing more: its peers' waits
+    // for its rows then expire and they abort in turn, so at most a phase or two of bytes
+    // reach a barrier this CTA no longer arms.
+    auto targets = [&]() -> unsigned { return G > 1 && !*abort_flag ? peers : 0u; };
+    // entry (r, j) of a phase's vector vec into every CTA that owns rows (to: targets())
+    auto send = [&](T* vec, uint64_t* bar, unsigned to, int j, int r, T v) {
         vec[r * NR + j] = v;
         if constexpr (G > 1) {
-            if (*abort_flag) return;
             const uint32_t a = smem_u32(vec + r * NR + j), mb = smem_u32(bar);
 #pragma unroll
             for (int pr = 0; pr < G; ++pr)
-                if (pr != g) st_async(peer_addr(a, pr), v, peer_addr(mb, pr));
+                if (to & (1u << pr)) st_async(peer_addr(a, pr), v, peer_addr(mb, pr));
         }
     };
     // an owner warp, once all its rows of a phase are stored here (all of its lanes)
@@ -389,6 +398,10 @@ k_band_wide(const BandBlock* __restrict__ blocks, const T* __restrict__ fac, con
     dep_wait();                                          // (the copies so far are of the factor)
     // every CTA of the cluster has armed its barriers before any st.async reaches it
     cluster_barrier<G>();
+    if (G > 1 && nrb == 0) {                             // (no copy issued either: it has no quads)
+        cluster_barrier<G>();
+        return;
+    }
 
     // One block: this warp's share times the vector vin (complete once phase `par` of
     // vector barrier `vb` has), its pieces to `part`.
@@ -500,17 +513,19 @@ k_band_wide(const BandBlock* __restrict__ blocks, const T* __restrict__ fac, con
         }
         if (J > 0) run_block(upper, vst, &vbar[2], (uint32_t)(uy++ & 1));           // O_J y_{J-1}
         T* vtb = vt + (ut & 1) * NR * WP;
+        unsigned to = targets();
 #pragma unroll
         for (int it = 0; it < NIT; ++it)
-            if (own[it]) send(vtb, &vbar[ut & 1], oj[it], orow[it], J > 0 ? pre[it] - psum(0, it) : pre[it]);
+            if (own[it]) send(vtb, &vbar[ut & 1], to, oj[it], orow[it], J > 0 ? pre[it] - psum(0, it) : pre[it]);
         arrive_local(&vbar[ut & 1]);
         run_block(lower, vtb, &vbar[ut & 1], (uint32_t)((ut >> 1) & 1));           // D_J t
         ++ut;
+        to = targets();
 #pragma unroll
         for (int it = 0; it < NIT; ++it)
             if (own[it]) {
                 const T y = psum(1, it);
-                if (J + 1 < c) send(vst, &vbar[2], oj[it], orow[it], y);             // read by O_{J+1}
+                if (J + 1 < c) send(vst, &vbar[2], to, oj[it], orow[it], y);             // read by O_{J+1}
                 const int row = J * W + orow[it];
                 if (row < m) out[row0 + row + oj[it] * ldo] = y;
             }
@@ -528,17 +543,19 @@ k_band_wide(const BandBlock* __restrict__ blocks, const T* __restrict__ fac, con
         }
         if (J < c - 1) run_block(lower, vst, &vbar[2], (uint32_t)(uy++ & 1));       // O_{J+1}^T x_{J+1}
         T* vtb = vt + (ut & 1) * NR * WP;
+        unsigned to = targets();
 #pragma unroll
         for (int it = 0; it < NIT; ++it)
-            if (own[it]) send(vtb, &vbar[ut & 1], oj[it], orow[it], J < c - 1 ? pre[it] - psum(1, it) : pre[it]);
+            if (own[it]) send(vtb, &vbar[ut & 1], to, oj[it], orow[it], J < c - 1 ? pre[it] - psum(1, it) : pre[it]);
         arrive_local(&vbar[ut & 1]);
         run_block(upper, vtb, &vbar[ut & 1], (uint32_t)((ut >> 1) & 1));           // D_J^T t
         ++ut;
+        to = targets();
 #pragma unroll
         for (int it = 0; it < NIT; ++it)
             if (own[it]) {
                 const T x = psum(0, it);
-                if (J > 0) send(vst, &vbar[2], oj[it], orow[it], x);                  // read by O_J^T
+                if (J > 0) send(vst, &vbar[2], to, oj[it], orow[it], x);                  // read by O_J^T
                 const int row = J * W + orow[it];
                 if (row < m) out[row0 + row + oj[it] * ldo] = base ? bs[it] - x : x;
             }
