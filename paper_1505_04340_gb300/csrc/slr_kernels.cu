@@ -17,6 +17,7 @@
 #include <vector>
 
 #include "slr_device.h"
+#include "slr_once.h"
 
 namespace slr {
 
@@ -2275,31 +2276,33 @@ cudaError_t launch_spmv_e(const DevOperator<T>& op, int32_t nI, const T* y, int6
     return spmv_cols<T>(nI, nrhs, op.e_rp, op.e_ci, op.e_v, y, ldy, nullptr, 0, out, ldo, st);
 }
 
-// Grid of a persistent solve on the current device: one CTA per SM (fewer if
-// no step has that many CTA tasks), 0 if the kernel cannot be co-resident.
-// Raises a kernel's dynamic shared-memory limit to the opt-in maximum less its
-// static shared memory, once per kernel (the limit is process-wide per kernel, so
-// it is never set per launch).  False if the device refuses.
+// Raises a kernel's dynamic shared-memory limit on the current device to the opt-in maximum
+// less its static shared memory, once per kernel and device (the limit is state of the
+// two, so it is never set per launch).  False if the device refuses.
 bool raise_smem_once(const void* kern) {
-    static std::mutex mu;
-    static std::vector<const void*> raised;
-    std::lock_guard<std::mutex> lk(mu);
-    if (std::find(raised.begin(), raised.end(), kern) != raised.end()) return true;
-    int dev = 0, optin = 0;
-    cudaFuncAttributes fa;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
-        cudaFuncGetAttributes(&fa, kern) != cudaSuccess ||
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             optin - (int)fa.sharedSizeBytes) != cudaSuccess) {
+    static OncePerDevice once;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
-    raised.push_back(kern);
-    return true;
+    return once.run(kern, dev, [&]() {
+        int optin = 0;
+        cudaFuncAttributes fa;
+        if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+            cudaFuncGetAttributes(&fa, kern) != cudaSuccess ||
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 optin - (int)fa.sharedSizeBytes) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        return true;
+    });
 }
 constexpr size_t kLevSmem = 200 * 1024;   // dynamic shared memory a per-level forward kernel may take
 
+// Grid of a persistent solve on the current device: one CTA per SM (fewer if
+// no step has that many CTA tasks), 0 if the kernel cannot be co-resident.
 template <typename K>
 int pers_grid(K kern, size_t smem, int32_t max_cta_tasks) {
     int dev = 0, nsm = 0, occ = 0;
