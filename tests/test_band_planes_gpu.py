@@ -52,3 +52,29 @@ def test_bsolve_at_tile_edges(W, c, skew, precision):
             block = t
         assert np.array_equal(t, block[:, :r]), r
     g.close()
+
+
+@pytest.mark.parametrize("W,c", [(65, 4), (96, 3), (128, 2), (224, 1), (225, 4), (255, 3), (257, 3)])
+@pytest.mark.parametrize("split,threads", [(1, 512), (1, 256), (2, 256), (4, 256), (4, 512)])
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_bsolve_of_wide_planes(W, c, split, threads, precision):
+    """The wider kernel at its first width and around whole row blocks, for each split and CTA size (a
+    slice holds at most 256 rows: the last width needs two)."""
+    if W > 256 and split == 1:
+        split = 2
+    P = problem(W, c, False)
+    order = dd_order(P.rowptr, P.colind, P.part, P.nparts)
+    f = np.random.default_rng(W).standard_normal((order.n_I, 11))
+    want = BSolver(split_blocks(P.rowptr, P.colind, P.val, order)[0], order.int_off).solve(f)
+    g = SLR(P.rowptr, P.colind, P.val, P.part, P.nparts, k=0, precision=precision, nrhs_max=11, band_split=split,
+            band_threads=threads)
+    info = g.get_info()
+    assert (info["band_split"], info["band_threads"]) == (split, threads)
+    tol = TOL64 if precision == "fp64" else tol32(info)
+    for r in (11, 7, 6, 5, 3, 2, 1):
+        t = g.bsolve(torch.tensor(f[:, :r], device="cuda")).cpu().numpy()
+        assert np.abs(t - want[:, :r]).max() <= tol * np.abs(want[:, :r]).max(), r
+        if r == 11:
+            block = t
+        assert np.array_equal(t, block[:, :r]), r
+    g.close()
