@@ -60,14 +60,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
         : "memory");
     return ok != 0;
 }
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-            smem_u32(dst)),
-        "l"(src), "r"(bytes), "r"(smem_u32(bar))
-        : "memory");
-}
-// The same with an L2 policy.  A factor larger than kL2Keep is read once per pass and gone
+// Bulk copy to shared memory with an L2 policy.  A factor larger than kL2Keep is read once per pass and gone
 // from L2 before the next one, so its lines are the first to leave and the vectors, which
 // the pass reads again, stay (FV 1024^2 FP32, a 378 MB factor: an apply takes 417 us with
 // the policy, 447 without); a factor that L2 can hold keeps the normal policy.
@@ -78,7 +71,7 @@ __device__ __forceinline__ uint64_t policy_stream(bool once) {
     else asm volatile("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(p));
     return p;
 }
-__device__ __forceinline__ void bulk_g2s_pol(void* dst, const void* src, uint32_t bytes, uint64_t* bar, uint64_t pol) {
+__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar, uint64_t pol) {
     asm volatile(
         "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;" ::"r"(
             smem_u32(dst)),
@@ -279,7 +272,7 @@ k_band_wide(const BandBlock* __restrict__ blocks, const T* __restrict__ fac, con
                             (itype == 0 ? 0 : itype == 1 ? SU : itype == 2 ? SU + SL : SU + 2 * SL);
         const uint32_t bytes = (uint32_t)(n * 128 * (int)sizeof(T));
         mbar_arrive_expect_tx(&full[islot], bytes);
-        bulk_g2s_pol(ring + (size_t)islot * slot, facg + off + ((up ? sq0[0] : sq0[1]) + iq) * 128, bytes,
+        bulk_g2s(ring + (size_t)islot * slot, facg + off + ((up ? sq0[0] : sq0[1]) + iq) * 128, bytes,
                      &full[islot], pol);
         ++issued;
         iq += n;

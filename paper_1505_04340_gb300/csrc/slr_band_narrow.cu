@@ -104,7 +104,7 @@ k_band_narrow(const BandBlock* __restrict__ blocks, const T* __restrict__ fac, c
                                 (type == 0 ? 0 : type == 1 ? SU : type == 2 ? SU + SL : SU + 2 * SL);
             const uint32_t bytes = (uint32_t)((type == 0 || type == 3 ? SU : SL) * (int)sizeof(T));
             mbar_arrive_expect_tx(&full[sl], bytes);
-            bulk_g2s_pol(ring + (size_t)sl * slot, fac0 + off, bytes, &full[sl], pol);
+            bulk_g2s(ring + (size_t)sl * slot, fac0 + off, bytes, &full[sl], pol);
             next_block(c, type, plane);
             ++issued;
             if (++sl == nslot) sl = 0;

@@ -44,6 +44,7 @@ namespace {
 
 constexpr int kBtThreads = 256;
 constexpr int kSub = 4096;                 // bytes of one sub-tile (128 rows x 32 bytes)
+constexpr int kStiles = 4;                 // sub-tiles of a ring slot
 constexpr long long kBtSpin = 1ll << 24;   // polls of a bounded wait
 
 template <int AB>
@@ -192,7 +193,7 @@ template <int AB, int NP>
 __global__ void __launch_bounds__(kBtThreads, NP <= 32 ? 2 : 1)
 k_band_tc(const BandTcBlock* __restrict__ blocks, const unsigned char* __restrict__ fac, const float* in,
           int64_t ldi, float* out, int64_t ldo, const float* base, int64_t ldb, int32_t nrhs, int32_t nslot,
-          int32_t stiles, int32_t* err) {
+          int32_t* err) {
     dep_go();
     dep_wait();
     using Tp = BtType<AB>;
@@ -207,8 +208,8 @@ k_band_tc(const BandTcBlock* __restrict__ blocks, const unsigned char* __restric
     // One operand buffer: a block's MMAs all complete (acc_bar) before its epilogue
     // overwrites the operand with the next block's, and the next block's MMAs wait
     // for that epilogue (opnd_bar), so the two never overlap.
-    unsigned char* ring = sm;                                      // nslot x stiles sub-tiles
-    unsigned char* vbuf = ring + (size_t)nslot * stiles * kSub;    // the vector operand
+    unsigned char* ring = sm;                                      // nslot x kStiles sub-tiles
+    unsigned char* vbuf = ring + (size_t)nslot * kStiles * kSub;    // the vector operand
     uint64_t* full = reinterpret_cast<uint64_t*>(vbuf + (size_t)vbytes);
     uint64_t* empty = full + nslot;
     uint64_t* acc_bar = empty + nslot;
@@ -268,19 +269,19 @@ k_band_tc(const BandTcBlock* __restrict__ blocks, const unsigned char* __restric
             const int nt = tiles_of(bk.type);
             const int64_t boff = bk.type == 0 ? 0 : bk.type == 1 ? nU : bk.type == 2 ? nU + nL : nU + 2 * nL;
             const unsigned char* src = fac + b.foff + ((int64_t)bk.plane * (2 * nU + 2 * nL) + boff) * kSub;
-            for (int t0 = 0; t0 < nt; t0 += stiles, ++f) {
+            for (int t0 = 0; t0 < nt; t0 += kStiles, ++f) {
                 if (f >= nslot && !tc::mbar_wait(&empty[s], par, kBtSpin)) {
                     fail();
                     break;
                 }
                 if (*abort_flag) break;
-                const uint32_t bytes = (uint32_t)(min(stiles, nt - t0) * kSub);
+                const uint32_t bytes = (uint32_t)(min(kStiles, nt - t0) * kSub);
                 asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(tc::smem_addr(&full[s])),
                              "r"(bytes)
                              : "memory");
                 asm volatile(
                     "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;" ::"r"(
-                        tc::smem_addr(ring + (size_t)s * stiles * kSub)),
+                        tc::smem_addr(ring + (size_t)s * kStiles * kSub)),
                     "l"(src + (int64_t)t0 * kSub), "r"(bytes), "r"(tc::smem_addr(&full[s])), "l"(pol)
                     : "memory");
                 if (++s == nslot) {
@@ -330,19 +331,19 @@ k_band_tc(const BandTcBlock* __restrict__ blocks, const unsigned char* __restric
                         break;
                     }
                     // the sub-tiles of this M-tile in the slot
-                    const int n = min(stiles - in_slot, k1 - ks);
-                    const uint64_t ad = ring_desc + kSubDesc * (uint32_t)(s * stiles + in_slot);
+                    const int n = min(kStiles - in_slot, k1 - ks);
+                    const uint64_t ad = ring_desc + kSubDesc * (uint32_t)(s * kStiles + in_slot);
                     const uint64_t bd = vec_desc + kStepDesc * (uint32_t)ks;
                     if (elected) {
                         tc::mma<AB>(d, ad, bd, idesc, ks > k0);
 #pragma unroll
-                        for (int i = 1; i < 8; ++i)
+                        for (int i = 1; i < kStiles; ++i)
                             if (i < n) tc::mma<AB>(d, ad + kSubDesc * i, bd + kStepDesc * i, idesc, true);
                     }
                     ks += n;
                     in_slot += n;
                     left -= n;
-                    if (in_slot == stiles || left == 0) {       // the slot's last sub-tile
+                    if (in_slot == kStiles || left == 0) {       // the slot's last sub-tile
                         if (elected) tc::commit(&empty[s]);
                         in_slot = 0;
                         if (++s == nslot) {
@@ -499,16 +500,15 @@ cudaError_t bt_launch(const DevOperator<float>& op, int32_t p, const float* in, 
     // with more subdomains than SMs, in half an SM (113 KB: two CTAs per SM, one wave).
     // 3-D 96^3, 32 columns, one B-solve with its two conversions: 522 us with five slots of
     // 16 KB, 526 with two of 32 KB, 529 with six of 12 KB.
-    const int stiles = 4;
     const size_t cap = (NP <= 32 && p > op.cf.nsm) ? 113 * 1024 : 227 * 1024;
-    int nslot = fixed < cap ? (int)((cap - fixed) / ((size_t)stiles * kSub)) : 0;
+    int nslot = fixed < cap ? (int)((cap - fixed) / ((size_t)kStiles * kSub)) : 0;
     nslot = nslot > 8 ? 8 : nslot;
     if (nslot < 2) return cudaErrorInvalidValue;
-    const size_t smem = (size_t)nslot * stiles * kSub + fixed;
+    const size_t smem = (size_t)nslot * kStiles * kSub + fixed;
     cudaError_t e = cudaFuncSetAttribute(k_band_tc<AB, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     if (e != cudaSuccess) return e;
     e = launch_dep(k_band_tc<AB, NP>, p, kBtThreads, smem, st, op.band_tc, op.band_tc_fac, in, ldi, out, ldo, base, ldb,
-                   nrhs, nslot, stiles, op.err);
+                   nrhs, nslot, op.err);
     count_launches(1);
     return e;
 }
