@@ -337,8 +337,8 @@ k_band_wide(const BandBlock* __restrict__ blocks, const T* __restrict__ fac, con
     // pass's last t and the backward pass's first t have no exchange of y
     // between them, so a fast peer can send the second before a slow CTA has
     // read the first.  y/x needs one buffer (an exchange of t always lies between
-    // two of its phases).  A slice without rows (planes of fewer than G row blocks)
-    // sends nothing that could hold its peers back: with their next bytes in a phase
+    // two of its phases).  A slice without rows (planes of fewer than G row blocks,
+    // or of few more, where the assignment leaves one out) sends nothing that could hold its peers back: with their next bytes in a phase
     // it has yet to arm, the phase's count never comes to zero.  So it takes no part: its peers
     // send it nothing and it waits for nothing.  After a wait that expired the barrier
     // is left un-armed (thread 0 never arrives twice in one phase).

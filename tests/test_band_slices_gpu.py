@@ -2,7 +2,8 @@
 give every CTA rows.
 
 Four subdomains whose planes are about ``narrow`` and ``wide`` rows wide: the split follows the
-widest, so the narrow ones' clusters have CTAs without a 32-row block.  Oracle, tolerances and the
+widest, so the narrow ones' clusters have CTAs without a 32-row block; at 192 rows the
+assignment of six blocks to four CTAs leaves one out.  Oracle, tolerances and the
 column's independence as in ``test_band_planes_gpu.py``.
 """
 import numpy as np
@@ -22,7 +23,7 @@ from paper_1505_04340_gb300 import SLR  # noqa: E402
 from tolerances import TOL64, tol32  # noqa: E402
 
 
-@pytest.mark.parametrize("narrow,wide", [(1, 128), (32, 200), (40, 200), (70, 129), (96, 257)])
+@pytest.mark.parametrize("narrow,wide", [(1, 128), (32, 200), (40, 200), (70, 129), (96, 257), (192, 192)])
 @pytest.mark.parametrize("split,threads", [(0, 0), (2, 512), (4, 256)])
 @pytest.mark.parametrize("precision", ["fp64", "mixed"])
 def test_bsolve_of_slices_without_rows(narrow, wide, split, threads, precision):
