@@ -97,8 +97,9 @@ typedef struct {
                                Must be SLR_U_FP32 with SLR_PREC_FP64                       */
 
     /* ---- execution choices: each gives the same preconditioner up to rounding; band_slots,
-       band_order and host_loop give bitwise the same result (band_split, band_threads and
-       c_persistent, which autotune picks too, set how some sums are split)              */
+       band_order and host_loop give bitwise the same result.  band_split, band_threads and
+       c_persistent set how some sums are split: handles that have to agree bit for bit fix
+       these three and leave autotune, which picks them by time, off                     */
     int32_t band_split;     /* CTAs (a thread-block cluster) per subdomain in the band solve:
                                1, 2 or 4; 0 = automatic                                  */
     int32_t band_slots;     /* shared-memory buffers the band solve streams its factor

@@ -202,7 +202,8 @@ slr_status upload_operator(slr_handle h, DevOperator<T>& op, bool with_band) {
         d.max_cta_tasks = std::max(d.max_cta_tasks, nt + np);
     }
     // fused levels stage a supernode's [L_JJ^{-1}; M_J] in shared memory when it fits
-    // 56 KB (three CTAs per SM beside their vectors: with 36 KB, FP64 3-D 64^3 took 1014 us
+    // 56 KB (beside their vectors three CTAs per SM; two in the backward kernel of blocks, whose
+    // vectors take 32 KB, 44 KB in FP64.  With 36 KB, FP64 3-D 64^3 took 1014 us
     // per apply, 996 now, the C solve of 16 columns on 75 x 70 x 81 641, 615 now), the persistent
     // kernels, four groups to a CTA, 36 KB each; the
     // forward stages the panel with an odd row stride (n_J | 1), so sizes count it
@@ -894,7 +895,10 @@ slr_status autotune(slr_handle h, DevOperator<T>& op, cudaStream_t st) {
                     }
                 }
         }
-        // the C solves run inside the PCG graph: time them as a replayed graph
+        // the C solves run inside the PCG graph: time them as a replayed graph.  (Outside a graph the
+        // per-level path has dependent launches, the persistent one not; on seven problems, 2-D 32^2 to
+        // 3-D 96^3, in both precisions with 1, 5 and 32 columns, either way of timing picked the
+        // same path: the persistent one in two of the 42 cases.)
         double c_us[2] = {0, 0};
         for (int v = 0; v < 2; ++v) {
             op.cf.per_level = (v == 0);
@@ -972,9 +976,12 @@ slr_status setup_impl(slr_handle h, int32_t n, const int32_t* rowptr, const int3
             // of 128 rows or more go four ways (two ways) while two 256-thread CTAs per SM
             // hold all slices, so that one slice's exchange hides behind the other's
             // products (W = 225, one column, CTAs per subdomain 1, 2, 4: 64 subdomains 564, 361,
-            // 327 us, 27: 563, 359, 240, 8: 421, 274, 223; W = 196, 125 subdomains: 422, 379, 422; W = 100, 64
-            // subdomains: 162, 124, 136).  FP32 takes two while each slice has an SM of its
-            // own, four if those have (64 subdomains 143, 102, 168 us; 27: 142, 99, 93; 8: 112, 89, 86).
+            // 327 us, 27: 563, 359, 241, 8: 563, 358, 237; W = 196, 125 subdomains: 422, 379, 422; W = 81 to
+            // 121, 64 subdomains: 162, 124, 137).  FP32 takes two while each slice has an SM of its
+            // own, four if those have (CTAs of 512 threads, W = 225: 64 subdomains 138, 98, 165 us; 27: 137, 95,
+            // 87; 8: 139, 95, 87).  At 64 subdomains four CTAs of 256 threads, two on an SM, take 95 us for
+            // one column but 346 against 312 for five and 384 against 326 for eight: the autotuner, which
+            // knows the block's width, picks them for one.
             const bool fp64 = h->opts.precision == SLR_PREC_FP64;
             if (wmx >= 128 && 4 * nparts <= (fp64 ? 2 * nsm : nsm)) G = 4;
             else if ((wmx >= 64 && 2 * nparts <= nsm) || (fp64 && wmx >= 128 && nparts <= nsm)) G = 2;

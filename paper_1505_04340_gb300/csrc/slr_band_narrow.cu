@@ -20,9 +20,9 @@
 // Results and right-hand sides move between a lane and global memory for the same
 // (column, right-hand side) in both passes, so the backward pass reads what its own
 // thread wrote; right-hand sides are loaded two planes ahead.
-// Measured: FV 1024^2 in 256 subdomains (W = 62, 62 planes), FP32: 140 us per B-solve,
-// 5.4 TB/s of DRAM traffic (the segments' padding included); one warp per subdomain
-// walking every segment in turn took 405 us.  2-D 32^2 (W = 15, FP64): 82 -> 42 us, bound
+// Measured: FV 1024^2 in 256 subdomains (W = 62, 62 planes), FP32: 131 us per B-solve, in which
+// the kernel moves 0.78 GB of DRAM traffic at 6.0 TB/s (the quads' padding included); one warp per
+// subdomain walking every segment in turn took 405 us.  2-D 32^2 (W = 15, FP64): 82 -> 40 us, bound
 // by the latency of 58 blocks' seven dependent FP64 operations each.
 //
 // Up to eight right-hand sides (FP64: four) share a launch (the factor is read once).  Each sums its

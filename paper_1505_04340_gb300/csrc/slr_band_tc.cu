@@ -8,7 +8,7 @@
 //   backward  t = Y_J - O_{J+1}^T X_{J+1},  X_J = D_J^T t
 // Each of the four products per plane is a dense W x W (triangular) block times
 // a W x r block, i.e. an MMA with M = W (one or two tiles of 128 rows), K = W
-// (steps of KS columns: 8 TF32 or 16 BF16) and N = r (padded to NP = 16, 32, 48
+// (steps of KS columns: 8 TF32 or 16 BF16) and N = r (padded to NP = 16, 32
 // or 64).  The factor is packed once (k_band_tc_pack) as "sub-tiles" of 128 rows
 // x KS columns, 4096 bytes each, already in the K-major core-matrix layout of
 // slr_tc.cuh (SBO = 256, LBO = 128), keeping only the sub-tiles that meet the
@@ -260,7 +260,10 @@ k_band_tc(const BandTcBlock* __restrict__ blocks, const unsigned char* __restric
 
     if (tid == 0) {
         // ---------------------------------------------------------------- producer
-        uint64_t pol;                                   // the factor leaves L2 first: it is read once per pass
+        // The factor leaves L2 first, also one that L2 could hold for the second B-solve: the vectors
+        // and the C factor gain more (apply of 16 columns with and without, us: 32^3 641, 654; 40^3 329,
+        // 336; 47^3 410, 413; 64^3 873, 879)
+        uint64_t pol;
         asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
         int f = 0, s = 0;                               // copies issued, slot of the next one
         uint32_t par = 1;                               // parity of the slot's last release
