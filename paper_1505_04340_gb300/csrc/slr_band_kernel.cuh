@@ -195,6 +195,7 @@ k_band_wide(const BandBlock* __restrict__ blocks, const T* __restrict__ fac, con
     uint64_t* full = reinterpret_cast<uint64_t*>(smem) + warp * kMaxBuf;   // [kW][kMaxBuf]
     uint64_t* vbar = reinterpret_cast<uint64_t*>(smem) + kW * kMaxBuf;      // [3] t (two buffers), y/x
     volatile int* abort_flag = reinterpret_cast<volatile int*>(vbar + 3);
+    volatile unsigned* dest = reinterpret_cast<volatile unsigned*>(abort_flag + 1);   // CTAs this one sends to
     int* R0s = reinterpret_cast<int*>(vbar + 4);                            // [kRB] first row of each row block
     int2* pw = reinterpret_cast<int2*>(R0s + kRB);                          // [2][kRB] first and last warp of a row
                                                                             // block (upper, lower)
@@ -248,6 +249,10 @@ k_band_wide(const BandBlock* __restrict__ blocks, const T* __restrict__ fac, con
         for (int i = 0; i < nbuf; ++i) mbar_init(&full[i], 1);
     if (tid == 0) {
         *abort_flag = 0;                                  // set once a bounded wait of this CTA expires
+        unsigned peers = 0;                               // the others that own rows
+        for (int pr = 0; pr < G; ++pr)
+            if (pr != g && b.nrb[pr] > 0) peers |= 1u << pr;
+        *dest = peers;
         for (int i = 0; i < 3; ++i) mbar_init(&vbar[i], 1 + narr);
         for (int i = 0; i < 3; ++i) {
             if (rbytes) mbar_arrive_expect_tx(&vbar[i], rbytes);
@@ -288,6 +293,7 @@ k_band_wide(const BandBlock* __restrict__ blocks, const T* __restrict__ fac, con
     // with whatever its buffers hold (no wait is taken again).
     auto fail = [&]() {
         atomicExch(err, 1);
+        *dest = 0;
         *abort_flag = 1;
     };
     int kslot = 0;                                        // slot and parity of the next copy to read
@@ -358,16 +364,11 @@ k_band_wide(const BandBlock* __restrict__ blocks, const T* __restrict__ fac, con
         }
         __syncwarp();
     };
-    unsigned peers = 0;                                   // the other CTAs that own rows
-    if constexpr (G > 1) {
-#pragma unroll
-        for (int pr = 0; pr < G; ++pr)
-            if (pr != g && b.nrb[pr] > 0) peers |= 1u << pr;
-    }
-    // The peers that a phase's rows go to.  An aborted CTA sends nothing more: its peers' waits
-    // for its rows then expire and they abort in turn, so at most a phase or two of bytes
-    // reach a barrier this CTA no longer arms.
-    auto targets = [&]() -> unsigned { return G > 1 && !*abort_flag ? peers : 0u; };
+    // The peers that a phase's rows go to: a word in shared memory, read once per phase (in a register
+    // it cost the eight-column kernel, which spills, 4%).  An aborted CTA sends nothing more: its
+    // peers' waits for its rows then expire and they abort in turn, so at most a phase or two of
+    // bytes reach a barrier this CTA no longer arms.
+    auto targets = [&]() -> unsigned { return G > 1 ? *dest : 0u; };
     // entry (r, j) of a phase's vector vec into every CTA that owns rows (to: targets())
     auto send = [&](T* vec, uint64_t* bar, unsigned to, int j, int r, T v) {
         vec[r * NR + j] = v;
