@@ -183,7 +183,6 @@ k_band_wide(const BandBlock* __restrict__ blocks, const T* __restrict__ fac, con
     const int g = (G > 1) ? (int)cg::this_cluster().block_rank() : 0;
     const BandBlock& b = blocks[sub];
     const int W = b.w, c = b.c, m = b.m, WP = (W + 3) & ~3;
-    dep_go();
     if (m == 0) {                               // uniform across the cluster
         dep_wait();
         return;

@@ -73,7 +73,6 @@ k_band_narrow(const BandBlock* __restrict__ blocks, const T* __restrict__ fac, c
     constexpr int PB = kNw * NR * 64;                  // partial sums of a block
     extern __shared__ __align__(128) unsigned char smem[];
     const int W = blocks[blockIdx.x].w, c = blocks[blockIdx.x].c, m = blocks[blockIdx.x].m;
-    dep_go();
     if (m == 0) {
         dep_wait();
         return;

@@ -194,7 +194,6 @@ __global__ void __launch_bounds__(kBtThreads, NP <= 32 ? 2 : 1)
 k_band_tc(const BandTcBlock* __restrict__ blocks, const unsigned char* __restrict__ fac, const float* in,
           int64_t ldi, float* out, int64_t ldo, const float* base, int64_t ldb, int32_t nrhs, int32_t nslot,
           int32_t* err) {
-    dep_go();
     dep_wait();
     using Tp = BtType<AB>;
     using Te = typename Tp::Te;

@@ -164,18 +164,22 @@ int64_t thread_launches();
 
 // Dependent launches.  An apply is a chain of 10 to 45 kernels of 4 to 40 us, and a plain launch
 // starts when the kernel before it has ended and its stores are flushed.  Within a DepScope a
-// kernel launched by launch_dep may start once every CTA of the one before has started: its
+// kernel launched by launch_dep may start once every CTA of the one before has exited: its
 // CTAs take their places, read what no kernel of the chain writes (the factors, index tables) and
 // stop at dep_wait until the kernel before has completed and its stores are visible.  Rules:
 //   every kernel launched by launch_dep calls dep_wait, and touches nothing that another kernel of
 //   the chain writes before it; since that kernel waited too, all before it have completed;
 //   such data are read by plain loads (no __restrict__ const or __ldg: a non-coherent load may
 //   see what the SM's L1 held before the wait);
+//   no kernel lets its dependents start before it ends (griddepcontrol.launch_dependents): their CTAs would
+//   take the room that is left, many on one SM, and stay there.  With that at every kernel's start an FP64 C
+//   solve of 32 columns on 3-D 32^3 took 692 us (434 with plain launches, 432 now), an FP64 apply of 8 columns
+//   on 2-D 357^2 1236 (1034, 1003), in FP32 236 (212 now);
 //   the scope opens after the chain's first kernel, launched plainly, so what ran before the chain is complete;
 //   not while the stream is captured: the graphs keep plain edges.
-// Measured (us per call, plain -> dependent): apply 2-D 32^2 FP64 123 -> 104, 3-D 64^3 mixed 413 -> 357 and
-// FP64 992 -> 958, FV 1024^2 383 -> 350, 32 columns of 3-D 96^3 2526 -> 2443; C solve of 16 columns on
-// 75 x 70 x 81 541 -> 474.
+// Measured (us per call, plain -> dependent): apply 2-D 32^2 FP64 123 -> 103, 3-D 64^3 mixed 413 -> 356 and
+// FP64 992 -> 942, FV 1024^2 383 -> 349, 32 columns of 3-D 96^3 2526 -> 2415; C solve of 16 columns on
+// 75 x 70 x 81 541 -> 479.
 class DepScope {
 public:
     explicit DepScope(cudaStream_t st, bool on = true);
@@ -190,8 +194,6 @@ bool dep_active();                  // the calling thread is in a DepScope
 
 #ifdef __CUDACC__
 __device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-// the next kernel of the chain may start once every CTA has come here
-__device__ __forceinline__ void dep_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <typename... P, typename... A>
 cudaError_t launch_dep(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {

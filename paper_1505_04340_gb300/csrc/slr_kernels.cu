@@ -112,7 +112,6 @@ template <typename T>
 __global__ void k_spmv_cols(int32_t rows, int32_t nrhs, const int32_t* __restrict__ rp,
                             const int32_t* __restrict__ ci, const T* __restrict__ v, const T* x, int64_t ldx,
                             const T* g, int64_t ldg, T* y, int64_t ldy) {
-    dep_go();
     dep_wait();
     const int32_t ngr = (nrhs + kSpCols - 1) / kSpCols;
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1394,7 +1393,6 @@ template <typename T, int NW>
 __global__ void __launch_bounds__(NW * 32, NW == 8 ? 4 : 1)
 k_cfwd_level(const CView<T> cf, int32_t t0, int32_t p0, int32_t np, const T* g, int64_t ldg, T* xf, int32_t nrhs,
              int32_t tstride, int32_t rbmax) {
-    dep_go();
     dep_wait();
     extern __shared__ __align__(16) unsigned char csm[];
     __shared__ T red[NW][33];
@@ -1413,7 +1411,6 @@ k_cfwd_level(const CView<T> cf, int32_t t0, int32_t p0, int32_t np, const T* g, 
 template <typename T, int NW, int RP, int R>
 __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 1)
 k_cfwd_level_blk(const CView<T> cf, int32_t t0, int32_t p0, int32_t np, T* xf, int32_t nrhs, int32_t tstride) {
-    dep_go();
     dep_wait();
     extern __shared__ __align__(16) unsigned char csm[];
     const int q = blockIdx.x, j0 = blockIdx.y * RP;
@@ -1430,7 +1427,6 @@ k_cfwd_level_blk(const CView<T> cf, int32_t t0, int32_t p0, int32_t np, T* xf, i
 template <typename T>
 __global__ void __launch_bounds__(256)
 k_cperm_g(int32_t s, int32_t nrhs, const int32_t* __restrict__ ciperm, const T* g, int64_t ldg, T* gf) {
-    dep_go();
     dep_wait();
     __shared__ T tile[32][33];
     const int i0 = blockIdx.x * 32, j0 = blockIdx.y * 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -1453,7 +1449,6 @@ k_cperm_g(int32_t s, int32_t nrhs, const int32_t* __restrict__ ciperm, const T* 
 template <typename T>
 __global__ void __launch_bounds__(256)
 k_cperm_y(int32_t s, int32_t nrhs, const int32_t* __restrict__ ciperm, const T* xf, T* y, int64_t ldy) {
-    dep_go();
     dep_wait();
     __shared__ T tile[32][33];
     const int i0 = blockIdx.x * 32, j0 = blockIdx.y * 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -1477,7 +1472,6 @@ k_cperm_y(int32_t s, int32_t nrhs, const int32_t* __restrict__ ciperm, const T* 
 template <typename T>
 __global__ void __launch_bounds__(256)
 k_cfwd_gather(const CView<T> cf, int32_t s0, const T* g, int64_t ldg, int32_t nrhs) {
-    dep_go();
     dep_wait();
     const int32_t J = cf.lev_sn[s0 + blockIdx.x];
     const int32_t a0 = cf.c0[J], nJ = cf.c0[J + 1] - a0;
@@ -1495,7 +1489,6 @@ k_cfwd_gather(const CView<T> cf, int32_t s0, const T* g, int64_t ldg, int32_t nr
 template <typename T, int NW>
 __global__ void __launch_bounds__(NW * 32, NW == 8 ? 4 : 1)
 k_cbwd_level(const CView<T> cf, int32_t t0, const T* yf, T* xf, T* y_dd, int64_t ldy, int32_t nrhs) {
-    dep_go();
     dep_wait();
     extern __shared__ __align__(16) unsigned char csm[];
     __shared__ T red[NW][33];
@@ -1511,7 +1504,6 @@ k_cbwd_level(const CView<T> cf, int32_t t0, const T* yf, T* xf, T* y_dd, int64_t
 template <typename T, int NW, int RP>
 __global__ void __launch_bounds__(NW * 32, NW == 8 ? 2 : 1)
 k_cbwd_level_blk(const CView<T> cf, int32_t t0, const T* yf, T* xf, T* y_dd, int64_t ldy, int32_t nrhs, int ystage) {
-    dep_go();
     dep_wait();
     extern __shared__ __align__(16) unsigned char csm[];
     T* us = reinterpret_cast<T*>(csm);
@@ -1533,7 +1525,6 @@ template <typename T, int RB, bool TILED>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 2)
 k_cfwd_small(const CView<T> cf, int32_t s0, const T* g, int64_t ldg, T* xf, int32_t nrhs, int32_t cap,
              int32_t tsz) {
-    dep_go();
     extern __shared__ __align__(16) unsigned char csm[];
     T* ts = reinterpret_cast<T*>(csm);
     cfwd_small_cta<T, kThreads, 1, RB, TILED>(cf, cf.lev_sn[s0 + blockIdx.x], ts, g, ldg, xf, nrhs, ts + tsz, cap);
@@ -1546,7 +1537,6 @@ template <typename T, int RB, bool TILED>
 __global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 3 : 2)
 k_cbwd_small(const CView<T> cf, int32_t s0, const T* yf, T* xf, T* y_dd, int64_t ldy, int32_t nrhs, int32_t cap,
              int32_t vsz) {
-    dep_go();
     extern __shared__ __align__(16) unsigned char csm[];
     T* vs = reinterpret_cast<T*>(csm);
     T* red = vs + RB * (kSmallN + kSmallR);
@@ -1586,7 +1576,6 @@ constexpr int kTopT = 256;   // threads of the zone kernels (8 warps)
 template <typename T>
 __global__ void __launch_bounds__(kThreads)
 k_ctop_gather(const CView<T> cf, const T* g, int64_t ldg, int32_t nrhs) {
-    dep_go();
     dep_wait();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (int64_t)cf.nT * nrhs) return;
@@ -1630,7 +1619,6 @@ constexpr int kTopR = sizeof(T) == 4 ? 8 : 4;
 template <typename T, int RB>
 __global__ void __launch_bounds__(kTopT)
 k_ctop_fwd(const CView<T> cf, T* xf, int32_t nrhs) {
-    dep_go();
     dep_wait();
     __shared__ T ts[RB][kTopCW];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1700,7 +1688,6 @@ k_ctop_fwd(const CView<T> cf, T* xf, int32_t nrhs) {
 template <typename T, int RB>
 __global__ void __launch_bounds__(kTopT)
 k_ctop_bwd(const CView<T> cf, const T* yf, T* xf, T* y_dd, int64_t ldy, int32_t nrhs) {
-    dep_go();
     dep_wait();
     constexpr int NW = kTopT / 32, DEPTH = sizeof(T) == 4 ? 16 : 8;
     __shared__ __align__(16) T xs[kTopRCH * RB];
@@ -1898,7 +1885,6 @@ __host__ __device__ inline int lr_blocks(int32_t s) {
 template <typename T>
 __global__ void __launch_bounds__(256)
 k_lr_vt(int32_t s, int32_t k, int32_t nrhs, const T* __restrict__ U, const T* w, int64_t ldw, T* part) {
-    dep_go();
     dep_wait();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int R = (s + gridDim.x - 1) / gridDim.x;
@@ -1951,7 +1937,6 @@ constexpr int kLrSeg = 16, kLrFinJ = 16;
 template <typename T>
 __global__ void __launch_bounds__(kLrSeg * kLrFinJ)
 k_lr_vt_fin(int32_t k, int32_t nrhs, int32_t G, const T* part, const T* __restrict__ dvec, T* vk) {
-    dep_go();
     dep_wait();
     __shared__ T seg[kLrSeg][kLrFinJ];
     const int kk = blockIdx.x, jl = threadIdx.x % kLrFinJ, q = threadIdx.x / kLrFinJ;
@@ -1983,7 +1968,6 @@ template <typename T, int JG>
 __global__ void __launch_bounds__(256)
 k_lr_update(int32_t s, int32_t k, int32_t nrhs, const T* __restrict__ U, const T* vk, T cinv, T* w,
             int64_t ldw) {
-    dep_go();
     dep_wait();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= s) return;
@@ -2023,7 +2007,6 @@ constexpr int kConvN = 4 * kThreads;
 template <typename TS, typename TD>
 __global__ void __launch_bounds__(kThreads)
 k_convert(int64_t rows, int32_t cols, const TS* src, int64_t lds, TD* dst, int64_t ldd) {
-    dep_go();
     dep_wait();
     const int64_t i0 = (int64_t)blockIdx.x * kConvN + threadIdx.x;
     for (int64_t j = blockIdx.y; j < cols; j += gridDim.y) {

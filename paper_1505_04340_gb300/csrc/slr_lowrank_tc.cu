@@ -63,7 +63,6 @@ template <int AB, int UK, int WK>
 __global__ void __launch_bounds__(kTcThreads, 1)
 k_lr_vt_tc(int32_t s, int32_t k, int32_t nrhs, int32_t np, const typename TcType<AB>::U* __restrict__ Ucm,
            const float* w, float* part, int32_t* err) {
-    dep_go();
     dep_wait();
     using Tp = TcType<AB>;
     using Te = typename Tp::U;
@@ -181,7 +180,6 @@ template <int AB>
 __global__ void __launch_bounds__(kTcThreads, 1)
 k_lr_update_tc(int32_t s, int32_t k, int32_t kp, int32_t nrhs, int32_t np, const typename TcType<AB>::U* __restrict__ Urm,
                const float* vk, float cinv, float* w, int32_t* err) {
-    dep_go();
     dep_wait();
     using Tp = TcType<AB>;
     using Te = typename Tp::U;
@@ -300,7 +298,6 @@ k_lr_update_tc(int32_t s, int32_t k, int32_t kp, int32_t nrhs, int32_t np, const
 constexpr int kFinSeg = 16, kFinJ = 16;
 __global__ void __launch_bounds__(kFinSeg * kFinJ)
 k_lr_fin_tc(int32_t k, int32_t nrhs, int32_t G, const float* part, const float* __restrict__ dvec, float* vk) {
-    dep_go();
     dep_wait();
     __shared__ float seg[kFinSeg][kFinJ];
     const int kk = blockIdx.x, j = blockIdx.y * kFinJ + (threadIdx.x % kFinJ), q = threadIdx.x / kFinJ;

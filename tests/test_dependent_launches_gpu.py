@@ -1,7 +1,7 @@
-"""Calls whose kernels start before the ones ahead of them have ended, against the same calls with plain edges.
+"""Calls whose kernels start before the stores of the ones ahead are flushed, against the same calls with plain edges.
 
 Outside stream capture the kernels of a call are dependent launches; a captured call has plain
-edges, so each kernel waits for the whole of the one before.  Calls back to back, each on what the
+edges.  Calls back to back, each on what the
 one before has just written, give bit for bit what the captured call gives on the same input.
 """
 import numpy as np
