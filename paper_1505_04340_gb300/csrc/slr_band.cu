@@ -50,7 +50,15 @@ cudaError_t launch_band_solve(const DevOperator<T>& op, int32_t p, int32_t wmax,
         const int nt = op.band_nt;
         int32_t nb, cq;
         auto fits = [&](int n) { return band_ring(wmax, n, sizeof(T), 0, nt, &nb, &cq) && nb * cq >= 6; };
-        const int nv = sizeof(T) == 4 && left > 4 && fits(8) ? 8 : left > 2 && fits(4) ? 4 : left > 1 && fits(2) ? 2 : 1;
+        // FP64: three columns in a kernel of their own, since its pipe takes the absent fourth's
+        // multiply-adds as well (B-solve of three columns on 3-D 60^3, 64 subdomains: 994 us by the kernel of
+        // four, 1007 for four; 838 as two and one with the earlier kernels; 721 now)
+        constexpr int three = sizeof(T) == 4 ? 4 : 3;
+        const int nv = sizeof(T) == 4 && left > 4 && fits(8) ? 8
+                       : left > 3 && fits(4)                 ? 4
+                       : left > 2 && fits(three)             ? three
+                       : left > 1 && fits(2)                 ? 2
+                                                             : 1;
         const int nr = std::min(nv, left);
         const T* bs = base ? base + c * ldb : nullptr;
         cudaError_t e = cudaSuccess;
@@ -60,12 +68,18 @@ cudaError_t launch_band_solve(const DevOperator<T>& op, int32_t p, int32_t wmax,
             if constexpr (sizeof(T) == 4) {
                 if (nv == 8) e = band_launch_half<T, 8>(op, p, wmax, ic, ldi, oc, ldo, bs, ldb, nr, st);
             }
+            if constexpr (sizeof(T) == 8) {
+                if (nv == 3) e = band_launch_half<T, 3>(op, p, wmax, ic, ldi, oc, ldo, bs, ldb, nr, st);
+            }
             if (nv == 4) e = band_launch_half<T, 4>(op, p, wmax, ic, ldi, oc, ldo, bs, ldb, nr, st);
             else if (nv == 2) e = band_launch_half<T, 2>(op, p, wmax, ic, ldi, oc, ldo, bs, ldb, nr, st);
             else if (nv == 1) e = band_launch_half<T, 1>(op, p, wmax, ic, ldi, oc, ldo, bs, ldb, nr, st);
         } else {
             if constexpr (sizeof(T) == 4) {
                 if (nv == 8) e = band_launch_g<T, 8, 512>(op, p, wmax, ic, ldi, oc, ldo, bs, ldb, nr, st);
+            }
+            if constexpr (sizeof(T) == 8) {
+                if (nv == 3) e = band_launch_g<T, 3, 512>(op, p, wmax, ic, ldi, oc, ldo, bs, ldb, nr, st);
             }
             if (nv == 4) e = band_launch_g<T, 4, 512>(op, p, wmax, ic, ldi, oc, ldo, bs, ldb, nr, st);
             else if (nv == 2) e = band_launch_g<T, 2, 512>(op, p, wmax, ic, ldi, oc, ldo, bs, ldb, nr, st);

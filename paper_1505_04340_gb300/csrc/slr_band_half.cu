@@ -20,6 +20,7 @@ SLR_HALF(float, 4)
 SLR_HALF(float, 8)
 SLR_HALF(double, 1)
 SLR_HALF(double, 2)
+SLR_HALF(double, 3)
 SLR_HALF(double, 4)
 #undef SLR_HALF
 

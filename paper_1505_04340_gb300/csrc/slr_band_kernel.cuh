@@ -429,7 +429,7 @@ k_band_wide(const BandBlock* __restrict__ blocks, const T* __restrict__ fac, con
                         for (int w = 0; w < U; ++w)
 #pragma unroll
                             for (int j = 0; j < NR; ++j)
-                                if (NR <= 2 || j < nr) {
+                                if (NR <= 3 || j < nr) {
                                     T& s = ((u + w) & 1) ? ac2[j] : acc[j];
                                     s = fma(a[u + w], v[w * NR + j], s);
                                 }
