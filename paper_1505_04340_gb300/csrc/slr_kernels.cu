@@ -1612,6 +1612,24 @@ __device__ __forceinline__ void last_task_sum(int32_t* cnt, int nch, const T* pa
 template <typename T>
 constexpr int kTopR = sizeof(T) == 4 ? 8 : 4;
 
+// The passes over nrhs right-hand sides: pass(width, first), whole ones of RB, then the rest.  In
+// FP64 the last pass has the rest's own width: absent columns would cost its pipe as much as
+// present ones (C solve of 5 columns on 3-D 47^3: 690 us with a second pass of four, 569 now).  FP32
+// has the room, and takes the rest in a pass of RB.
+template <typename T, int RB, typename F>
+__device__ __forceinline__ void top_passes(int32_t nrhs, F pass) {
+    int j0 = 0;
+    for (; j0 + RB <= nrhs; j0 += RB) pass(std::integral_constant<int, RB>{}, j0);
+    if (j0 == nrhs) return;
+    if constexpr (sizeof(T) == 8 && RB == 4) {
+        if (nrhs - j0 == 3) pass(std::integral_constant<int, 3>{}, j0);
+        else if (nrhs - j0 == 2) pass(std::integral_constant<int, 2>{}, j0);
+        else pass(std::integral_constant<int, 1>{}, j0);
+    } else {
+        pass(std::integral_constant<int, RB>{}, j0);
+    }
+}
+
 // forward task (row block rb, columns [cb, ce), chunk k): partial sums of rows
 // r0 .. r0 + count - 1 of L_TT^{-1} t_T over the chunk for RB right-hand sides at a time; a warp
 // takes rows w, w + 8, w + 16, w + 24 (four in flight), lanes over the columns; the 4 x RB sums
@@ -1632,17 +1650,18 @@ k_ctop_fwd(const CView<T> cf, T* xf, int32_t nrhs) {
         la[u] = r < rb.y ? rb.x + r : -1;
         off[u] = r < rb.y ? cf.tsk_off[la[u]] - cf.tsk_lo[la[u]] : 0;
     }
-    for (int j0 = 0; j0 < nrhs; j0 += RB) {
-        const int nb = min(RB, nrhs - j0);
+    top_passes<T, RB>(nrhs, [&](auto width, int j0) {
+        constexpr int NB = decltype(width)::value, NP = NB == 3 ? 4 : NB;   // NP: a power of two
+        const int nb = min(NB, nrhs - j0);
 #pragma unroll
-        for (int b = 0; b < RB; ++b) {
+        for (int b = 0; b < NB; ++b) {
             const T* t = cf.tT + (int64_t)(j0 + min(b, nb - 1)) * cf.nT;
             for (int c = tk.y + threadIdx.x; c < tk.z; c += kTopT) ts[b][c - tk.y] = t[c];
         }
         __syncthreads();
-        T acc[4 * RB];
+        T acc[4 * NP];
 #pragma unroll
-        for (int q = 0; q < 4 * RB; ++q) acc[q] = T(0);
+        for (int q = 0; q < 4 * NP; ++q) acc[q] = T(0);
         int c = tk.y + lane;
         // sixteen loads in flight per lane (four rows x four columns); entries right
         // of a row's diagonal, and rows past the block, load nothing
@@ -1655,10 +1674,10 @@ k_ctop_fwd(const CView<T> cf, T* xf, int32_t nrhs) {
 #pragma unroll
             for (int q = 0; q < 4; ++q)
 #pragma unroll
-                for (int b = 0; b < RB; ++b) {
+                for (int b = 0; b < NB; ++b) {
                     const T tv = ts[b][c + 32 * q - tk.y];
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) acc[u * RB + b] += a[u][q] * tv;
+                    for (int u = 0; u < 4; ++u) acc[u * NP + b] += a[u][q] * tv;
                 }
         }
         for (; c < tk.z; c += 32) {
@@ -1667,16 +1686,16 @@ k_ctop_fwd(const CView<T> cf, T* xf, int32_t nrhs) {
                 if (c <= la[u]) {
                     const T a = cf.tsk[off[u] + c];
 #pragma unroll
-                    for (int b = 0; b < RB; ++b) acc[u * RB + b] += a * ts[b][c - tk.y];
+                    for (int b = 0; b < NB; ++b) acc[u * NP + b] += a * ts[b][c - tk.y];
                 }
         }
         __syncwarp();
-        const T v = reduce_scatter<T, 4 * RB>(acc, lane);
-        const int k = rs_index<4 * RB>(lane), u = k / RB, b = k % RB;
-        if (rs_writer<4 * RB>(lane) && b < nb && warp + 8 * u < rb.y)
+        const T v = reduce_scatter<T, 4 * NP>(acc, lane);
+        const int k = rs_index<4 * NP>(lane), u = k / NP, b = k % NP;
+        if (rs_writer<4 * NP>(lane) && b < nb && warp + 8 * u < rb.y)
             cf.tf_part[(int64_t)(j0 + b) * cf.tf_parts + rb.w + tk.w * 32 + warp + 8 * u] = v;
         __syncthreads();
-    }
+    });
     last_task_sum(cf.tf_cnt + tk.x, rb.z, cf.tf_part + rb.w, cf.tf_parts, rb.y, nrhs,
                   [&](int r, int j, T v) { xf[cf.tpos[rb.x + r] + (int64_t)j * cf.s] = v; });
 }
@@ -1700,23 +1719,24 @@ k_ctop_bwd(const CView<T> cf, const T* yf, T* xf, T* y_dd, int64_t ldy, int32_t 
     const int32_t* pp = cf.tp_pos + cf.tp_off[J];
     const int nrw = tk.z - tk.y, per = (nrw + NW - 1) / NW;
     const int rb = tk.y + warp * per, re = min(tk.z, rb + per);
-    for (int j0 = 0; j0 < nrhs; j0 += RB) {
-        const int nb = min(RB, nrhs - j0);
+    top_passes<T, RB>(nrhs, [&](auto width, int j0) {
+        constexpr int NB = decltype(width)::value;
+        const int nb = min(NB, nrhs - j0);
         for (int r = tk.y + threadIdx.x; r < tk.z; r += kTopT) {
             const T* y = yf + pp[r] + (int64_t)j0 * cf.s;
 #pragma unroll
-            for (int b = 0; b < RB; ++b) xs[(r - tk.y) * RB + b] = b < nb ? y[(int64_t)b * cf.s] : T(0);
+            for (int b = 0; b < NB; ++b) xs[(r - tk.y) * NB + b] = b < nb ? y[(int64_t)b * cf.s] : T(0);
         }
         __syncthreads();
-        T acc[RB];
+        T acc[NB];
 #pragma unroll
-        for (int b = 0; b < RB; ++b) acc[b] = T(0);
+        for (int b = 0; b < NB; ++b) acc[b] = T(0);
         if (lane < cb.z) {
             auto madd = [&](T a, int r) {
-                const T* x = xs + (r - tk.y) * RB;
+                const T* x = xs + (r - tk.y) * NB;
 #pragma unroll
-                for (int q = 0; q < RB; q += RB < 4 ? 1 : 4) {
-                    if constexpr (RB < 4) {
+                for (int q = 0; q < NB; q += NB < 4 ? 1 : 4) {
+                    if constexpr (NB < 4) {
                         acc[q] += a * x[q];
                     } else {
                         T t4[4];
@@ -1737,7 +1757,7 @@ k_ctop_bwd(const CView<T> cf, const T* yf, T* xf, T* y_dd, int64_t ldy, int32_t 
             for (; r < re; ++r) madd(X[(int64_t)r * nJ], r);
         }
 #pragma unroll
-        for (int b = 0; b < RB; ++b) red[warp][b][lane] = acc[b];
+        for (int b = 0; b < NB; ++b) red[warp][b][lane] = acc[b];
         __syncthreads();
         for (int b = warp; b < nb; b += NW)
             if (lane < cb.z) {
@@ -1747,7 +1767,7 @@ k_ctop_bwd(const CView<T> cf, const T* yf, T* xf, T* y_dd, int64_t ldy, int32_t 
                 cf.tb_part[(int64_t)(j0 + b) * cf.tb_parts + pofs + tk.w * 32 + lane] = v;
             }
         __syncthreads();
-    }
+    });
     const int32_t a0 = cf.c0[J] + cb.y;
     last_task_sum(cf.tb_cnt + tk.x, cb.w, cf.tb_part + pofs, cf.tb_parts, cb.z, nrhs, [&](int c, int j, T v) {
         xf[(int64_t)(a0 + c) * cf.xr + j] = v;

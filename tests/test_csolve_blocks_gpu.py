@@ -55,3 +55,18 @@ def test_applies_in_a_row_equal_applies_alone(precision, nrhs, side):
             torch.cuda.synchronize()
             assert torch.equal(x, y)
     g.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("nrhs", [2, 3, 5, 6, 7, 11])
+def test_csolve_last_pass_widths_equal_single_columns(precision, nrhs):
+    """Widths whose last pass over the top levels' inverse is narrower than the ones before: every column
+    equals the column solved alone, bit for bit."""
+    P = slrgen.make_problem("m32", (32, 32, 32), (2, 2, 2), 4)
+    g = SLR(P.rowptr, P.colind, P.val, P.part, P.nparts, k=0, precision=precision, nrhs_max=nrhs)
+    assert g.get_info()["c_top_positions"] > 0
+    gg = np.random.default_rng(nrhs).standard_normal((g.s, nrhs))
+    y = g.csolve(cu(gg)).cpu().numpy()
+    for c in range(nrhs):
+        assert np.array_equal(g.csolve(cu(gg[:, c])).cpu().numpy(), y[:, c]), c
+    g.close()
