@@ -483,7 +483,7 @@ def kernel_roofline(kind, info, prec, nrhs, us, hbm, hbm_src, name):
     if kind == "band":        # one B-solve: forward and backward pass over the band factor
         entries = info["band_entries"]
         vec = 2 * info["n_interior"] * nrhs * wf
-        label = "k_band_wide (K1, one B-solve)"
+        label = f"k_band_{'narrow' if info['band_threads'] == 32 else 'wide'} (K1, one B-solve)"
     else:                     # one C-solve: L^{-1} then L^{-T} (diagonal blocks, panels, top-zone inverse)
         entries = info["c_diag_entries"] + info["c_panel_entries"] + info["c_top_entries"]
         vec = 4 * info["s"] * nrhs * wf
